@@ -789,7 +789,7 @@ int create_impl(const spider_catalog* cat, const spider_stations* sta, const spi
   if (scr) {
     if ((e = dalloc(L, &c->tt_scratch, scr))) return bail(cuda_fail(c, e, "alloc scratch"));
   }
-  if ((e = configure_step_kernels(v))) return bail(cuda_fail(c, e, "kernel attributes"));
+  if ((e = configure_step_kernels())) return bail(cuda_fail(c, e, "kernel attributes"));
   c->pgrid = pcg_grid(v, c->num_sms);
   if (c->pgrid < 1) {
     c->err = "whitening kernel does not fit on the device (block too large)";

@@ -1800,11 +1800,18 @@ cudaError_t launch_select(const StepView& v, int64_t n_b, cudaStream_t st, int b
 size_t resid_smem(const StepView& v) { return (size_t)(3 * v.L_max + 2 * v.B) * sizeof(float); }
 size_t final_smem(const StepView& v) { return (size_t)(2 * v.L_max + v.B) * sizeof(float); }
 
-cudaError_t configure_step_kernels(const StepView& v) {
+// The limits of the per-block kernels are those of the largest block there can
+// be (4096 observations of 8192 local nodes), whatever this context needs: they
+// belong to the kernels, and a context with smaller blocks must not lower them
+// for an older one.
+cudaError_t configure_step_kernels() {
+  constexpr int kObs = 4096, kNodes = 2 * kObs;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(k_resid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)resid_smem(v))))
+  if ((e = cudaFuncSetAttribute(k_resid, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)((3 * kNodes + 2 * kObs) * sizeof(float)))))
     return e;
-  if ((e = cudaFuncSetAttribute(k_final, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)final_smem(v))))
+  if ((e = cudaFuncSetAttribute(k_final, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)((2 * kNodes + kObs) * sizeof(float)))))
     return e;
   if ((e = cudaFuncSetAttribute(k_comp_solve, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)(kCompWarps * sizeof(WarpSmem)))))
