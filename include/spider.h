@@ -273,20 +273,18 @@ int spider_last_timing(spider_ctx *ctx, float out_ms[5], int64_t *pairs,
  * (CUDA events on the context stream; zeros while timing is off):
  * out[0] selection + pair table, [1] travel times, [2] residuals and u = B^T r
  * (k_resid), [3] merge of u over blocks sharing a pair (k_merge_rhs),
- * [4] whitening solve (matrix, components, solvers), [5] q = Sigma^-1 r and
+ * [4] whitening solve (components, solvers), [5] q = Sigma^-1 r and
  * per-node sums (k_final), [6] scaled dlogp/dT onto pairs (k_merge_s),
  * [7] centroid, [8] priors + update per event (k_event), [9] log posterior.
  * *touched_events: events with at least one pair in the minibatch. */
 int spider_last_kernel_timing(spider_ctx *ctx, float out_ms[10], int64_t *touched_events);
 
-/* Phases of the whitening solve of the last timed evaluation, when it took
- * the piece-inverse path (all zero otherwise; synchronous): [0] labelling the
- * selected pieces and grouping them into units, [1] the units' set-up (their
- * shared nodes, the pieces' (A_p[G,G])^-1 and S^-1), [2] the units' Schur
- * rounds and convergence check, [3] the CTA passes for units beyond the
- * data-parallel limits, [4] waiting for the clean-piece solver on its side
- * stream, [5] the general component solver (a no-op unless a unit exceeded
- * every limit).  Device ms from CUDA events. */
+/* Phases of the whitening solve of the last timed evaluation (all zero without
+ * whitening; synchronous): [0] labelling the selected pieces and listing the
+ * components, [1] zero, [2] the components held by one warp or one CTA (what
+ * they take beyond [3]), [3] the components spread over several CTAs,
+ * [4] waiting for the clean-piece solver on its branch stream, [5] pieces whose
+ * stored inverse did not converge.  Device ms from CUDA events. */
 int spider_last_whiten_timing(spider_ctx *ctx, float out_ms[6]);
 
 /* Debug views of the last evaluation (synchronous):
@@ -299,21 +297,21 @@ int spider_debug_obs(spider_ctx *ctx, int64_t *idx_out, float *r_out, float *q_o
 
 /* Launch-shape knobs that change speed but not results (every pair and every
  * connected component is computed independently of how work is spread):
- * knobs[0] CTAs per SM-slot of the per-component warp solver (1..8),
- * knobs[1] of the per-component CTA solver (1..4), knobs[2] CTAs per SM of
- * the FP32 MLP kernel (1..2), knobs[3] 1 (default): minibatch steps whiten
- * through the precomputed inverses of the block-local components when they
- * were built, 0: always through the general component solver; knobs[4]
- * (0..4, default 2) the share, in quarters, of the persistent grid the
- * clean-piece solver takes on its side stream while the units are solved
- * (0: it runs after them on the context's stream); knobs[5] (1, 2 (default)
- * or 4) threads per CTA of the per-block kernels (pair table, residuals,
- * whitened residuals), in units of 256 (the observations and nodes each thread
- * handles; changes only the rounding order of the FP64 log-likelihood sum);
- * knobs[6] 1 (default): the size classes of the units' small inverses
- * (piece blocks, then Schur complements) run side by side on four branch
- * streams, 0: one after the other on the context's stream.  The first
- * min(n, 7) knobs are set, the others kept.  Invalidates the captured step graph. */
+ * knobs[0] CTAs per SM-slot of the components held by one warp (1..8),
+ * knobs[1] of those held by one CTA (1..4), knobs[2] CTAs per SM of
+ * the FP32 MLP kernel (1..2), knobs[3] 1 (default): a piece (a block-local
+ * component) that shares no node with another selected block is solved with
+ * its stored inverse, where the inverses were built, 0: every component by
+ * conjugate gradients; knobs[4] (0..4, default 2) the share, in quarters, of
+ * the persistent grid the stored inverses' kernel takes on its branch stream
+ * (0: it runs after the other components on the context's stream); knobs[5]
+ * (1, 2 (default) or 4) threads per CTA of the per-block kernels (pair table,
+ * residuals, whitened residuals), in units of 256 (the observations and nodes
+ * each thread handles; changes only the rounding order of the FP64
+ * log-likelihood sum); knobs[6] 1 (default): the size classes of the
+ * components run side by side on branch streams, 0: one after the other on the
+ * context's stream.  The first min(n, 7) knobs are set, the others kept.
+ * Invalidates the captured step graph. */
 int spider_set_tuning(spider_ctx *ctx, const int32_t *knobs, int32_t n);
 
 /* Facts about a context (synchronous), out[0..n): [0] sub-problems,
@@ -322,18 +320,12 @@ int spider_set_tuning(spider_ctx *ctx, const int32_t *knobs, int32_t n);
  * [6] observations, [7] connected components of the last minibatch graph,
  * [8] block-local nodes (occurrences of pairs in blocks) in total,
  * [9] 1 if the inverses of the block-local components were precomputed,
- * [10] 1 if minibatch steps whiten through them, [11] units of pieces that
- * shared nodes in the last such step, [12] 1 if that step fell back to the
- * general component solver (a unit beyond the limits of the direct path),
- * [13] units of that step solved by the last unit pass, [14], [15] SM cycles /
- * 1024 spent on the units of the CTA pass and of the last pass, [16..30]
- * five counters per unit pass ([16..20] stay zero; [21..25] the CTA pass,
- * [26..30] the last pass): SM cycles / 1024 in set-up, the pieces' small
- * inverses, the inverse of S, the refinement rounds, and the units solved; [31..37] units the data-parallel unit solver handed to
- * the CTA passes since the context was created, by reason: too many pieces,
- * shared occurrences, shared nodes, shared nodes of one piece, a failed small
- * inverse, a failed inverse of S, a full pool; [38] kernel launches in the
- * captured step graph (0 until a graph step ran). */
+ * [10] 1 if pieces that share no node are solved with them, [11] components
+ * of the last whitening solve left to conjugate gradients, [12] 1 if one of
+ * them was spread over several CTAs (more than 1024 unique pairs or pieces),
+ * or a stored inverse did not converge, [13] components spread over several
+ * CTAs, [14..37] zero, [38] kernel launches in the captured step graph (0
+ * until a graph step ran). */
 int spider_info(spider_ctx *ctx, int64_t *out, int32_t n);
 
 /* Sampler diagnostics of Sec. 3.6 at the current state, accumulated in FP64 on

@@ -2,14 +2,13 @@
 
 Times every candidate setting of the knobs of `spider_set_tuning` (warp- and
 CTA-solver grid multipliers, FP32 MLP CTAs per SM, the clean-piece solver's
-share of the grid beside the units, the residual kernels' CTA size) on a live context for a few SGLD steps,
+share of the grid beside the other components, the residual kernels' CTA size) on a live context for a few SGLD steps,
 keeps the fastest, and caches it per workload signature in a JSON
 file (SPIDER_TUNE_CACHE, default ~/.cache/spider_gb300/tuning.json).  The knobs
 change speed only: results are identical for every setting.  The chain state is
-restored afterwards, so tuning does not advance the sampler.  Knob 6 (the size
-classes of the units' small inverses side by side on branch streams) is not
-swept and keeps its value (default on: 0.635 -> 0.49 ms of unit set-up on the
-1M-event step)."""
+restored afterwards, so tuning does not advance the sampler.  Knob 6 (the
+components' size classes side by side on branch streams) is not swept and keeps
+its value (default on)."""
 from __future__ import annotations
 
 import json

@@ -27,7 +27,7 @@ struct spider_ctx {
   StepView v{};
   std::vector<void*> allocs;
   float* tt_scratch = nullptr;
-  int gu = 0, pgrid = 0;
+  int gu = 0;
   int tag = 0;
   int64_t step = 0;
   int n_sub = 1;
@@ -38,15 +38,10 @@ struct spider_ctx {
   bool graph_ok = true;
   bool use_graph = true;
   int32_t knobs[7] = {2, 1, 2, 1, 2, 2, 1};   // see spider_set_tuning
-  // whitening through precomputed piece inverses (minibatch steps)
-  bool fast = false;               // tables built
-  bool mb_full_sub = false;        // a sub-problem selects all its blocks in a minibatch
-  int cc_grid = 0, clean_grid = 0;
-  int unit_grids[4] = {0, 0, 0, 0};   // [3]: SMs (the data-parallel unit solver)
-  int64_t piece_bytes = 0;
-  cudaStream_t side = nullptr;     // second stream of the piece-inverse whitening
-  cudaEvent_t fork = nullptr, join = nullptr;
-  Branches ubr{};                  // branch streams of the units' set-up
+  // whitening: grids of its kernels, the branch streams of its size classes
+  WhitenPlan plan{};
+  bool inv = false;                // the pieces' inverses were built
+  Branches ubr{};
   int64_t n_samples = 0;           // samples written so far (ring of sample_cap)
   int64_t last_nb = 0;
   bool timing = false;
@@ -59,7 +54,7 @@ struct spider_ctx {
   // centroid, k_event, end
   static constexpr int kEv = 11;
   cudaEvent_t ev[kEv] = {};
-  cudaEvent_t wev[5] = {};          // whitening phases (timed evaluations of the piece path)
+  cudaEvent_t wev[4] = {};          // whitening phases (timed evaluations)
   bool have_wtiming = false;
   int64_t graph_kernels = 0;        // kernel nodes of the captured step graph
   float last_ms[5] = {0, 0, 0, 0, 0};
@@ -84,7 +79,7 @@ int cuda_fail(spider_ctx* c, cudaError_t e, const char* what) {
 }
 
 void destroy_branches(Branches& b) {
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < kBranches; ++i) {
     if (b.s[i]) {
       cudaStreamSynchronize(b.s[i]);
       cudaStreamDestroy(b.s[i]);
@@ -235,9 +230,7 @@ int check_device_error(spider_ctx* c) {
 }
 
 // The kernels of one evaluation, in stream order (everything a step does).
-// fast: whiten through the piece inverses, with the general component solver
-// gated on the flag that path raises for units beyond its limits.
-cudaError_t step_sequence(spider_ctx* c, int64_t n_b, bool logpost, bool timed, bool fast) {
+cudaError_t step_sequence(spider_ctx* c, int64_t n_b, bool logpost, bool timed) {
   StepView& v = c->v;
   cudaStream_t st = c->stream;
   cudaError_t e;
@@ -265,16 +258,13 @@ cudaError_t step_sequence(spider_ctx* c, int64_t n_b, bool logpost, bool timed, 
   TRY(launch_tt(c->net, src, out, c->num_sms, c->tt_scratch, st, c->knobs[2]));
   if (timed) TRY(cudaEventRecord(c->ev[2], st));
   TRY(launch_resid(v, n_b, c->gu, st, timed ? &c->ev[3] : nullptr, 256 * c->knobs[5]));
-  if (fast) {
-    TRY(launch_whiten_fast(v, n_b, c->cfg.pcg_tol, c->cc_grid, c->unit_grids, c->clean_grid, st, c->side,
-                           c->fork, c->join, timed ? c->wev : nullptr, c->knobs[4],
-                           c->knobs[6] ? &c->ubr : nullptr));
-    StepView vg = v;
-    vg.gate = v.wfast + kWGeneral;
-    TRY(launch_pcg(vg, n_b, c->cfg.pcg_max_it, c->cfg.pcg_tol, c->pgrid, c->knobs[0], c->knobs[1], st));
-  } else {
-    TRY(launch_pcg(v, n_b, c->cfg.pcg_max_it, c->cfg.pcg_tol, c->pgrid, c->knobs[0], c->knobs[1], st));
-  }
+  WhitenPlan w = c->plan;
+  w.use_inv = c->inv && c->knobs[3];
+  w.clean_share = c->knobs[4];
+  w.warp_mult = c->knobs[0];
+  w.cta_mult = c->knobs[1];
+  TRY(launch_whiten(v, n_b, w, c->cfg.pcg_max_it, c->cfg.pcg_tol, st, c->knobs[6] ? &c->ubr : nullptr,
+                    timed ? c->wev : nullptr));
   if (timed) TRY(cudaEventRecord(c->ev[5], st));
   TRY(launch_finish(v, n_b, c->gu, logpost, st, timed ? &c->ev[6] : nullptr, 256 * c->knobs[5]));
 #undef TRY
@@ -288,7 +278,6 @@ int evaluate(spider_ctx* c, uint64_t seed, int mode, float eps) {
   const bool batch_full = cfg.batch_n <= 0 || cfg.batch_n >= v.N;
   const bool full = batch_full || (mode == 0 && seed == 0);
   const int64_t n_b = full ? c->nb_full : c->nb_mb;
-  const bool fast = c->fast && c->knobs[3] && !full && !c->mb_full_sub && v.whiten;
   cudaStream_t st = c->stream;
   StepParams hp{};
   hp.seed = seed;
@@ -312,7 +301,7 @@ int evaluate(spider_ctx* c, uint64_t seed, int mode, float eps) {
     // capture the step once; relaunch it every step with fresh parameters
     cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-      const cudaError_t e1 = step_sequence(c, n_b, false, false, fast);
+      const cudaError_t e1 = step_sequence(c, n_b, false, false);
       cudaGraph_t g = nullptr;
       const cudaError_t e2 = cudaStreamEndCapture(st, &g);
       if (e1 == cudaSuccess && e2 == cudaSuccess && g &&
@@ -344,7 +333,7 @@ int evaluate(spider_ctx* c, uint64_t seed, int mode, float eps) {
   if (graphable && c->graph_exec) {
     CK(c, cudaGraphLaunch(c->graph_exec, st));
   } else {
-    const cudaError_t e = step_sequence(c, n_b, mode == 0, c->timing, fast);
+    const cudaError_t e = step_sequence(c, n_b, mode == 0, c->timing);
     if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
   }
   if (c->timing) CK(c, cudaEventRecord(c->ev[spider_ctx::kEv - 1], st));
@@ -354,7 +343,7 @@ int evaluate(spider_ctx* c, uint64_t seed, int mode, float eps) {
   }
   c->last_nb = n_b;
   c->have_timing = c->timing;
-  c->have_wtiming = c->timing && fast;
+  c->have_wtiming = c->timing && v.whiten;
   return SPIDER_OK;
 }
 
@@ -396,35 +385,19 @@ void spider_config_default(spider_config* c) {
 
 namespace {
 
-// Pieces of every block and their inverses (pieces.h), for whitening the
-// minibatch steps; skipped (the general component solver serves every step)
-// when a piece is larger than the device path takes or the inverses would use
-// more than half of the free device memory.  Returns an error code only for a
-// failed CUDA call.
-int build_fast_whitening(spider_ctx* c, const Prep& P) {
+// The pieces of every block (pieces.h) and the tables of the whitening solve.
+// want_inverses: also the pieces' inverses, with which minibatch steps solve
+// the pieces that share no node; left out (conjugate gradients serve every
+// component) when a piece is larger than their kernel takes or they would use
+// more than half of the free device memory.
+int build_whitening(spider_ctx* c, const Prep& P, bool want_inverses) {
   Pieces T;
-  if (!build_pieces(P, piece_max_nodes(), &T, 0)) return SPIDER_OK;
-  const int64_t inv_floats = T.piece_inv_off[T.G];
-  const int64_t bytes = inv_floats * 4 + P.Q * (2 + 2 + 2 + 4 + 4) + P.N * 2 * 6 + (T.G + 1) * (8 + 4 * 7) +
-                        (P.NB + 1) * 4 +
-                        (int64_t)c->num_sms * whiten_unit_scratch_floats() * 4;
-  size_t free_b = 0, total_b = 0;
-  cudaError_t e = cudaMemGetInfo(&free_b, &total_b);
-  if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemGetInfo");
-  if (bytes > (int64_t)(free_b / 2)) return SPIDER_OK;
-  // the shared-memory attribute first: the occupancy query depends on it
-  if (configure_whiten_kernels() != cudaSuccess) {
-    cudaGetLastError();            // this device cannot run the direct path: the general solver serves
-    return SPIDER_OK;
-  }
-  c->cc_grid = piece_cc_grid(c->num_sms);
-  c->clean_grid = whiten_clean_grid(c->num_sms);
-  if (c->cc_grid < 1 || whiten_units_grids(c->num_sms, c->unit_grids) < 1 || c->clean_grid < 1) return SPIDER_OK;
-  c->unit_grids[3] = c->num_sms;
+  build_pieces(P, INT32_MAX, &T, 0);
   auto& L = c->allocs;
   StepView& v = c->v;
   cudaStream_t st = c->stream;
-  const size_t G = T.G, Q = P.Q;
+  cudaError_t e;
+  const size_t G = T.G, Q = P.Q, PP = P.P;
 #define UPF(field, src, n)                                                                       \
   do {                                                                                           \
     using _T = std::remove_const_t<std::remove_pointer_t<decltype(v.field)>>;                    \
@@ -444,43 +417,55 @@ int build_fast_whitening(spider_ctx* c, const Prep& P) {
   UPF(node_ppos, T.node_ppos.data(), Q);
   UPF(piece_node_off, T.piece_node_off.data(), G + 1);
   UPF(piece_nodes, T.piece_nodes.data(), Q);
-  UPF(piece_inv_off, T.piece_inv_off.data(), G + 1);
   UPF(mem_rp, T.mem_rp.data(), Q + 1);
   UPF(edge_pos, T.edge_pos.data(), T.edge_pos.size());
   UPF(edge_sw, T.edge_sw.data(), T.edge_sw.size());
   ALF(owner_b, Q);
-  ALF(plab, G);
-  ALF(pmulti, G);
-  ALF(pcount, G);
-  ALF(unit_of, G);
-  ALF(unit_cnt, G);
-  ALF(unit_off, G + 1);
-  ALF(unit_pieces, G);
-  ALF(unit_pblk, G);
-  ALF(unit_defer, G);
-  ALF(unit_defer2, G);
-  {
-    // the data-parallel unit solver: at most L_max occurrences per selected block
-    const size_t cap = (size_t)std::max<int64_t>(1, c->nb_mb) * (size_t)P.L_max;
-    v.u_cap = (int64_t)cap;
-    v.ginv_cap = int64_t(1) << 25;
-    v.sinv_cap = int64_t(1) << 24;
-    ALF(u_nocc, G); ALF(uocc_off, G + 1); ALF(u_ng, G); ALF(u_m, G);
-    ALF(u_gsz, G); ALF(u_goff, G + 1); ALF(u_ssz, G); ALF(u_soff, G + 1);
-    ALF(pu_base, G); ALF(pu_unit, G); ALF(pu_gb, G); ALF(pu_gn, G); ALF(pu_ginv, G);
-    ALF(o_g, cap); ALF(o_pe, cap); ALF(o_base, cap); ALF(o_u, cap); ALF(o_x, cap); ALF(o_unit, cap);
-    ALF(o_t, cap); ALF(o_i, cap);
-    ALF(o_uh, cap); ALF(o_ul, cap); ALF(o_zh, cap); ALF(o_zl, cap); ALF(o_f, cap); ALF(o_w, cap);
-    ALF(o_ph, cap); ALF(o_pl, cap);
-    ALF(sh_slot, cap); ALF(sh_sorted, cap); ALF(sh_tt, cap);
-    ALF(g_u, cap); ALF(g_beg, cap); ALF(g_cnt, cap);
-    ALF(g_uh, cap); ALF(g_ul, cap); ALF(g_zh, cap); ALF(g_zl, cap); ALF(g_f, cap); ALF(g_x, cap);
-    ALF(ginv_pool, (size_t)v.ginv_cap); ALF(sinv_pool, (size_t)v.sinv_cap);
-  }
+  ALF(plab, G); ALF(prow, G); ALF(pmulti, G); ALF(pcount, G); ALF(urows, G);
+  ALF(unit_of, G); ALF(unit_off, G); ALF(unit_np, G); ALF(unit_fill, G); ALF(unit_rows, G);
+  ALF(unit_slot, G);
+  ALF(msync, 2 * kMaxGrid);
+  ALF(unit_pieces, G); ALF(unit_pblk, G); ALF(unit_prow, G); ALF(unit_pbase, G);
+  ALF(cls_list, (size_t)kLists * G);
+  v.cls_cap = (int64_t)G;
   ALF(clean_list, G);
   ALF(clean_blk, G);
-  ALF(wfast, kWSlots + 64 + 32);
-  ALF(wscratch, (size_t)c->unit_grids[2] * whiten_unit_scratch_floats());
+  ALF(wfast, kWSlots + 64);
+  if ((e = cudaMemsetAsync(v.wfast, 0, (kWSlots + 64) * sizeof(int32_t), st))) return cuda_fail(c, e, "memset");
+  ALF(rowof, PP);
+  ALF(mrow, Q);
+  // entries of the largest step: two per selected observation, at most as much padding
+  ALF(ent, 4 * (size_t)P.N);
+  {
+    // rows of the multi-CTA class in whole slices: such a unit has more than
+    // kCtaRows rows, or more than kCtaPieces pieces
+    const size_t cap = PP + PP / 32 + G / 32 + 64;
+    ALF(rs_u, cap); ALF(rs_m, cap); ALF(rs_pm, cap); ALF(rs_len, cap); ALF(rs_slice, cap / 32 + 1);
+    ALF(rs_y, cap); ALF(rs_r, cap); ALF(rs_p, cap); ALF(rs_ap, cap); ALF(rs_dz, cap); ALF(rs_di, cap);
+    ALF(rs_zh, cap); ALF(rs_zl, cap);
+  }
+  if ((e = configure_solve_kernels())) return cuda_fail(c, e, "kernel attributes");
+  c->plan.num_sms = c->num_sms;
+  c->plan.cc_grid = components_grid(c->num_sms);
+  c->plan.clean_grid = whiten_clean_grid(c->num_sms);
+  c->plan.multi_grid = solve_multi_grid(c->num_sms);
+  if (c->plan.cc_grid < 2 || c->plan.clean_grid < 1 || c->plan.multi_grid < 1) {
+    c->err = "whitening kernels do not fit on the device";
+    return SPIDER_E_UNSUPPORTED;
+  }
+  if ((e = cudaEventCreateWithFlags(&c->ubr.fork, cudaEventDisableTiming))) return cuda_fail(c, e, "event");
+  for (int i = 0; i < kBranches; ++i) {
+    if ((e = cudaStreamCreateWithFlags(&c->ubr.s[i], cudaStreamNonBlocking))) return cuda_fail(c, e, "branch stream");
+    if ((e = cudaEventCreateWithFlags(&c->ubr.join[i], cudaEventDisableTiming))) return cuda_fail(c, e, "event");
+  }
+  // the host tables above must outlive the uploads
+  if ((e = cudaStreamSynchronize(st))) return cuda_fail(c, e, "upload sync");
+  if (!want_inverses || T.max_n > piece_max_nodes()) return SPIDER_OK;
+  const int64_t inv_floats = T.piece_inv_off[T.G];
+  size_t free_b = 0, total_b = 0;
+  if ((e = cudaMemGetInfo(&free_b, &total_b))) return cuda_fail(c, e, "cudaMemGetInfo");
+  if (inv_floats * 4 > (int64_t)(free_b / 2)) return SPIDER_OK;
+  UPF(piece_inv_off, T.piece_inv_off.data(), G + 1);
 #undef UPF
 #undef ALF
   float* inv = nullptr;
@@ -504,16 +489,7 @@ int build_fast_whitening(spider_ctx* c, const Prep& P) {
     b0 = b1;
   }
   if ((e = cudaStreamSynchronize(st))) return cuda_fail(c, e, "upload sync");
-  if ((e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking))) return cuda_fail(c, e, "side stream");
-  if ((e = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming))) return cuda_fail(c, e, "event");
-  if ((e = cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming))) return cuda_fail(c, e, "event");
-  if ((e = cudaEventCreateWithFlags(&c->ubr.fork, cudaEventDisableTiming))) return cuda_fail(c, e, "event");
-  for (int i = 0; i < 4; ++i) {
-    if ((e = cudaStreamCreateWithFlags(&c->ubr.s[i], cudaStreamNonBlocking))) return cuda_fail(c, e, "branch stream");
-    if ((e = cudaEventCreateWithFlags(&c->ubr.join[i], cudaEventDisableTiming))) return cuda_fail(c, e, "event");
-  }
-  c->piece_bytes = bytes;
-  c->fast = true;
+  c->inv = true;
   return SPIDER_OK;
 }
 
@@ -536,9 +512,6 @@ int create_impl(const spider_catalog* cat, const spider_stations* sta, const spi
       if (ev) cudaEventDestroy(ev);
     for (auto& ev : c->wev)
       if (ev) cudaEventDestroy(ev);
-    if (c->side) cudaStreamDestroy(c->side);
-    if (c->fork) cudaEventDestroy(c->fork);
-    if (c->join) cudaEventDestroy(c->join);
     destroy_branches(c->ubr);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;
@@ -627,7 +600,6 @@ int create_impl(const spider_catalog* cat, const spider_stations* sta, const spi
       const int64_t want = bfull ? nbs : std::min<int64_t>(nbs, (cfg->batch_n + P.B - 1) / P.B);
       sel_full[s2 + 1] = sel_full[s2] + (int32_t)nbs;
       sel_mb[s2 + 1] = sel_mb[s2] + (int32_t)want;
-      if (!bfull && want == nbs && nbs > 1) c->mb_full_sub = true;
       nobs[s2] = (int32_t)(P.sub_obs_off[s2 + 1] - P.sub_obs_off[s2]);
       nev[s2] = (int32_t)(P.sub_ev_off[s2 + 1] - P.sub_ev_off[s2]);
       ch[s2] = sub_chain[s2];
@@ -701,35 +673,7 @@ int create_impl(const spider_catalog* cat, const spider_stations* sta, const spi
   AL(diag, PP);
   AL(z, PP);
   AL(z_lo, PP);
-  AL(rres, PP);
-  AL(dz, PP);
-  AL(res, PP);
-  AL(pv, PP);
-  AL(pv2, PP);
   AL(umulti, PP);
-  AL(rowlen, PP);
-  AL(rowptr, PP + 1);
-  AL(occ_off, Q);
-  AL(csr_col, 2 * N);
-  AL(csr_sw, 2 * N);
-  AL(scan_part, kMaxGrid + 1);
-  AL(lab, PP);
-  AL(cslot, PP);
-  AL(ccount, PP);
-  AL(comp_root, PP);
-  AL(comp_off, PP + 1);
-  AL(members, PP + 1);
-  AL(lidx, PP);
-  AL(big, PP);
-  AL(chist, 512);
-  AL(cc_lroot, Q);
-  AL(bigpos, PP + 1);
-  AL(biglist, PP);
-  AL(corder, PP);
-  AL(centries, PP);
-  AL(ctier, PP);
-  AL(Ap, PP);
-  AL(yv, PP);
   AL(s_u, PP);
   AL(gp, PP);
   AL(pstamp, PP);
@@ -790,13 +734,8 @@ int create_impl(const spider_catalog* cat, const spider_stations* sta, const spi
     if ((e = dalloc(L, &c->tt_scratch, scr))) return bail(cuda_fail(c, e, "alloc scratch"));
   }
   if ((e = configure_step_kernels())) return bail(cuda_fail(c, e, "kernel attributes"));
-  c->pgrid = pcg_grid(v, c->num_sms);
-  if (c->pgrid < 1) {
-    c->err = "whitening kernel does not fit on the device (block too large)";
-    return bail(SPIDER_E_UNSUPPORTED);
-  }
-  if (v.whiten && !(cfg->batch_n <= 0 || cfg->batch_n >= (int64_t)N)) {
-    rc = build_fast_whitening(c, P);
+  if (v.whiten) {
+    rc = build_whitening(c, P, !(cfg->batch_n <= 0 || cfg->batch_n >= (int64_t)N));
     if (rc) return bail(rc);
   }
   c->ev_old = std::move(P.ev_old);
@@ -804,7 +743,7 @@ int create_impl(const spider_catalog* cat, const spider_stations* sta, const spi
   c->th0 = std::move(P.th0);
   for (int i = 0; i < spider_ctx::kEv; ++i)
     if ((e = cudaEventCreate(&c->ev[i]))) return bail(cuda_fail(c, e, "event"));
-  for (int i = 0; i < 5; ++i)
+  for (int i = 0; i < 4; ++i)
     if ((e = cudaEventCreate(&c->wev[i]))) return bail(cuda_fail(c, e, "event"));
   if ((e = cudaStreamSynchronize(st))) return bail(cuda_fail(c, e, "create sync"));
   *out = c;
@@ -1194,9 +1133,11 @@ int spider_last_whiten_timing(spider_ctx* c, float out_ms[6]) {
   CK(c, cudaStreamSynchronize(c->stream));
   for (int i = 0; i < 6; ++i) out_ms[i] = 0.f;
   if (!c->have_wtiming) return SPIDER_OK;
-  const cudaEvent_t a[6] = {c->ev[4], c->wev[0], c->wev[1], c->wev[2], c->wev[3], c->wev[4]};
-  const cudaEvent_t b[6] = {c->wev[0], c->wev[1], c->wev[2], c->wev[3], c->wev[4], c->ev[5]};
-  for (int i = 0; i < 6; ++i) CK(c, cudaEventElapsedTime(&out_ms[i], a[i], b[i]));
+  CK(c, cudaEventElapsedTime(&out_ms[0], c->ev[4], c->wev[0]));
+  CK(c, cudaEventElapsedTime(&out_ms[2], c->wev[2], c->wev[1]));
+  CK(c, cudaEventElapsedTime(&out_ms[3], c->wev[0], c->wev[2]));
+  CK(c, cudaEventElapsedTime(&out_ms[4], c->wev[1], c->wev[3]));
+  CK(c, cudaEventElapsedTime(&out_ms[5], c->wev[3], c->ev[5]));
   return SPIDER_OK;
 }
 
@@ -1266,16 +1207,14 @@ int spider_info(spider_ctx* c, int64_t* out, int32_t n) {
   int32_t cnt[kCntSlots] = {0};
   CK(c, cudaMemcpyAsync(cnt, c->v.counters, sizeof(cnt), cudaMemcpyDeviceToHost, c->stream));
   CK(c, cudaStreamSynchronize(c->stream));
-  int32_t wf[kWSlots + 64 + 32] = {0};
-  if (c->fast) {
+  int32_t wf[kWSlots] = {0};
+  if (c->v.wfast) {
     CK(c, cudaMemcpyAsync(wf, c->v.wfast, sizeof(wf), cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
   }
   int64_t vals[39] = {c->n_sub, c->graph_exec ? 1 : 0, c->nb_mb, c->nb_full, c->v.P, c->v.M, c->v.N,
-                      cnt[kCntComps], c->v.Q, c->fast ? 1 : 0, c->fast ? (c->mb_full_sub ? 0 : 1) : 0,
-                      wf[kWUnits], wf[kWGeneral], wf[kWBigS], wf[kWCycSm], wf[kWCycBig]};
-  for (int i = 0; i < 15; ++i) vals[16 + i] = wf[kWSlots + 64 + i];
-  for (int i = 0; i < 7; ++i) vals[31 + i] = wf[kWSlots + 64 + 16 + i];
+                      cnt[kCntComps], c->v.Q, c->inv ? 1 : 0, c->inv && c->knobs[3] ? 1 : 0,
+                      wf[kWUnits], wf[kWGeneral], wf[kWClass0 + kClsMulti]};
   vals[38] = c->graph_kernels;
   for (int32_t i = 0; i < n && i < 39; ++i) out[i] = vals[i];
   return SPIDER_OK;
@@ -1333,12 +1272,6 @@ void spider_destroy(spider_ctx* c) {
     if (e) cudaEventDestroy(e);
   if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
   if (c->graph) cudaGraphDestroy(c->graph);
-  if (c->side) {
-    cudaStreamSynchronize(c->side);
-    cudaStreamDestroy(c->side);
-  }
-  if (c->fork) cudaEventDestroy(c->fork);
-  if (c->join) cudaEventDestroy(c->join);
   destroy_branches(c->ubr);
   free_all(c->allocs);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);

@@ -25,15 +25,12 @@ cudaError_t mlp_tc_prepare(const float* W1_host, const float* const Wn_host[3], 
 
 // step (k_step.cu)
 cudaError_t configure_step_kernels();
-int pcg_grid(const StepView& v, int num_sms);
 cudaError_t launch_select(const StepView& v, int64_t n_b, cudaStream_t st, int bthreads = 256);
 // bthreads: threads per CTA of the per-block kernels k_resid and k_final (a
 // multiple of 32 up to 1024; results do not depend on it except the rounding
 // order of the FP64 r.q sums)
 cudaError_t launch_resid(const StepView& v, int64_t n_b, int gu, cudaStream_t st, const cudaEvent_t* ev,
                          int bthreads = 256);
-cudaError_t launch_pcg(const StepView& v, int64_t n_b, int max_it, float tol, int grid, int warp_mult,
-                       int cta_mult, cudaStream_t st);
 cudaError_t launch_finish(const StepView& v, int64_t n_b, int gu, bool logpost, cudaStream_t st,
                           const cudaEvent_t* ev, int bthreads = 256);
 // theta_0 + state (or a stored sample) in FP64, caller order (M x 4)
@@ -42,33 +39,35 @@ cudaError_t launch_state_out(const StepView& v, const float4* src, double* out, 
 cudaError_t launch_grad_out(const StepView& v, float4* out, int grid, cudaStream_t st);
 cudaError_t launch_diag(const StepView& v, const float4* g, const float4* G, double* norms, double* part,
                         int grid, cudaStream_t st);
-// whitening through the precomputed piece inverses (k_whiten.cu)
+// whitening (k_whiten.cu: components of the step, stored piece inverses;
+// k_solve.cu: conjugate gradients on the other components)
 int piece_max_nodes();
-int64_t whiten_unit_scratch_floats();   // global scratch per CTA of the unit solver
-cudaError_t configure_whiten_kernels();
-int whiten_units_grids(int num_sms, int grids[3]);
-int piece_cc_grid(int num_sms);
+int components_grid(int num_sms);
 int whiten_clean_grid(int num_sms);
+int solve_multi_grid(int num_sms);
+cudaError_t configure_solve_kernels();
 // branch streams on which independent kernels of one stage run side by side:
 // `fork` is recorded on the launching stream and waited on by each branch,
 // join[i] is recorded on branch i and waited on by the launching stream
+constexpr int kBranches = 5;
 struct Branches {
-  cudaStream_t s[4];
+  cudaStream_t s[kBranches];
   cudaEvent_t fork;
-  cudaEvent_t join[4];
+  cudaEvent_t join[kBranches];
 };
-// the units of a step, data-parallel (k_units.cu); br (nullable): the size
-// classes of the small inverses run concurrently on its streams
-cudaError_t launch_units(const StepView& v, float tol, int num_sms, cudaStream_t st, cudaEvent_t mid = nullptr,
-                         const Branches* br = nullptr);
-cudaError_t configure_units_kernels();
-// ev (nullable): five events recorded on st after the piece labelling, the
-// units' set-up, their refinement rounds, the CTA unit passes and the join
-// with the clean-piece solver (timed evaluations only)
-cudaError_t launch_whiten_fast(const StepView& v, int64_t n_b, float tol, int cc_grid, const int grids[4],
-                               int clean_grid, cudaStream_t st, cudaStream_t side, cudaEvent_t fork,
-                               cudaEvent_t join, const cudaEvent_t* ev = nullptr, int clean_share = 4,
-                               const Branches* br = nullptr);
+struct WhitenPlan {
+  int use_inv;                 // clean pieces through their stored inverses
+  int num_sms, cc_grid, clean_grid, multi_grid;
+  int clean_share;             // quarters of clean_grid on the branch stream (0: on the launching stream)
+  int warp_mult, cta_mult;     // CTAs per SM of the one-warp class / of the CTA classes
+};
+// ev (nullable): four events recorded after the components, the one-warp and
+// one-CTA classes, the multi-CTA class, and the join with the clean pieces
+// (timed evaluations only); br null: everything in turn on st
+cudaError_t launch_whiten(const StepView& v, int64_t n_b, const WhitenPlan& w, int max_it, float tol,
+                          cudaStream_t st, const Branches* br, const cudaEvent_t* ev);
+cudaError_t launch_solve_class(const StepView& v, int cls, int max_it, float tol, int ctas, cudaStream_t st);
+cudaError_t launch_solve_multi(const StepView& v, int max_it, float tol, int grid, cudaStream_t st);
 // stage-1 outlier mask (k_outlier.cu)
 size_t outlier_scratch_bytes(int n_sub);
 cudaError_t launch_outlier(const StepView& v, int n_sub, float kmad, void* scratch, uint8_t* keep,

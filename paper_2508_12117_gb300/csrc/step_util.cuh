@@ -117,12 +117,6 @@ __device__ __forceinline__ bool aborted(const StepView& v) {
   return *((volatile const int32_t*)v.counters + kCntError) != 0;
 }
 
-// In a step solved through the piece inverses, the general component solver
-// runs only when a unit exceeded the limits of that path (v.gate set).
-__device__ __forceinline__ bool gated_off(const StepView& v) {
-  return v.gate && *((volatile const int32_t*)v.gate) == 0;
-}
-
 // the same test taken once per CTA, for kernels with block-wide barriers
 __device__ __forceinline__ bool aborted_cta(const StepView& v) {
   __shared__ int a;

@@ -142,37 +142,7 @@ struct StepView {
   float* diag;       // lambda + diag(B^T B)
   float* z;          // solution (hi)
   float* z_lo;       //          (lo)
-  float* rres;       // outer (double-float) residual rounded to FP32: inner right-hand side
-  float* dz;         // inner correction
-  float* res;
-  float* pv;        // search direction (two buffers, alternating per iteration)
-  float* pv2;
-  float* Ap;
-  float* yv;
   uint8_t* umulti;  // per unique pair: 1 if it has occurrences in several selected blocks
-  // merged minibatch matrix lambda I + B^T B as CSR over unique pairs (per solve)
-  int32_t* rowlen;   // [P] half-edges of the pair over all selected occurrences
-  int32_t* rowptr;   // [P + 1]
-  int32_t* occ_off;  // [Q] offset of an occurrence's entries inside its pair's row
-  int32_t* csr_col;  // [2N] neighbour pair (unique index)
-  float* csr_sw;     // [2N] sqrt(w_e) of the edge
-  int32_t* scan_part;  // [kMaxGrid + 1] scan partials
-  // connected components of the minibatch graph (per solve)
-  int32_t* lab;      // [P] component label = smallest unique index in the component
-  int32_t* cslot;    // [P] per root: component index; per member: position (scratch)
-  int32_t* ccount;   // [P] member count per root
-  int32_t* comp_root;  // [P] roots in ascending order
-  int32_t* comp_off;   // [P + 1] member list offsets
-  int32_t* members;    // [P] member lists (sorted within each component by the solver)
-  int32_t* lidx;       // [P] local index of a member inside its component
-  uint8_t* big;        // [P] 1: the row belongs to a component solved by the grid-wide CG
-  int32_t* chist;      // [kCqBins + 4] solver work-list bins and cursors
-  int32_t* bigpos;     // [P + 1] exclusive prefix of the grid-tier flags (then the count)
-  int32_t* biglist;    // [P] grid-tier nodes in pair order
-  int32_t* cc_lroot;   // [Q] per local node of a selected block: its block-local component root (local node id)
-  int32_t* corder;     // [P] solver work list (component ids)
-  int32_t* centries;   // [P] CSR entries per component
-  uint8_t* ctier;      // [P] per component: 0 one warp, 1 one CTA, 2 grid-wide
   float* s_u;
   float4* gp;
   int32_t* pstamp;
@@ -183,46 +153,41 @@ struct StepView {
   double* dblk;      // FP64 sum r^2 per selected block (NB)
   double* dred;      // FP64 diagnostics partials, 4 x kMaxGrid
   double* dout;      // FP64 results: [0] loglik (scaled), [1] logprior, [2] logcen, [3] logpost
-  // whitening through the precomputed piece inverses (null when not built)
+  // pieces of every block (k_whiten.cu, k_solve.cu; null without whitening)
   const int32_t* blk_piece_off;   // NB + 1
   const uint16_t* node_piece;     // Q: piece of a local node, numbered within its block
   const uint16_t* node_ppos;      // Q: position of a local node inside its piece
   const int32_t* piece_node_off;  // G + 1
   const uint16_t* piece_nodes;    // Q: block-local index of each piece member
-  const int64_t* piece_inv_off;   // G + 1
-  const float* piece_inv;         // (lambda I + B^T B)^-1 of every piece, n x n each
   const int32_t* mem_rp;          // Q + 1: edges of each member (piece_nodes order)
   const uint16_t* edge_pos;       // 2N: position of the other end inside the piece
   const float* edge_sw;           // 2N: sqrt w of the edge
-  int32_t* owner_b;               // Q: block of the owner occurrence (per step)
-  int32_t* plab;                  // G: piece labels of the selected pieces (per step)
+  const int64_t* piece_inv_off;   // G + 1 (null when the inverses were not built)
+  const float* piece_inv;         // (lambda I + B^T B)^-1 of every piece, n x n each
+  // components of the step
+  int32_t* owner_b;               // Q: block of the owner occurrence
+  int32_t* plab;                  // G: piece labels
+  int32_t* prow;                  // G: owner occurrences of the piece
   uint8_t* pmulti;                // G: the piece has a node shared with another selected block
-  int32_t* pcount;                // G: pieces per unit, at the unit's root piece
+  int32_t* pcount;                // G: pieces of the component, at its root piece
+  int32_t* urows;                 // G: rows of the component, at its root piece
   int32_t* unit_of;               // G: unit of a root piece
-  int32_t* unit_cnt;              // [G]: pieces per unit (fill cursor afterwards)
-  int32_t* unit_off;              // [G + 1]
-  int32_t* unit_pieces;           // [G]
-  int32_t* unit_pblk;             // [G]: block of each entry of unit_pieces
-  int32_t* unit_defer;            // [G]: units the data-parallel solver handed to the CTA pass
-  int32_t* unit_defer2;           // [G]: units deferred from the CTA pass to the last pass
-  int32_t* clean_list;            // [G]: pieces of the step with no shared node
-  int32_t* clean_blk;             // [G]: their blocks
-  int32_t* wfast;                 // [kWSlots] unit count, unit cursor, fallback flag, rounds
-  float* wscratch;                // per CTA of the unit solver: S^-1 and the pieces' small inverses
-  // units solved data-parallel (k_units.cu): per unit [G (+1)], per unit piece
-  // entry [G], per occurrence slot [u_cap], pools of the small inverses
-  int32_t *u_nocc, *uocc_off, *u_ng, *u_m, *u_gsz, *u_goff, *u_ssz, *u_soff;
-  int32_t *pu_base, *pu_unit, *pu_gb, *pu_gn, *pu_ginv;
-  int32_t *o_g, *o_pe, *o_base, *o_u, *o_x, *o_unit, *o_t;
-  uint16_t* o_i;
-  float *o_uh, *o_ul, *o_zh, *o_zl, *o_f, *o_w, *o_ph, *o_pl;
-  int32_t *sh_slot, *sh_sorted;
-  float* sh_tt;
-  int32_t *g_u, *g_beg, *g_cnt;
-  float *g_uh, *g_ul, *g_zh, *g_zl, *g_f, *g_x;
-  float *ginv_pool, *sinv_pool;
-  int64_t u_cap, ginv_cap, sinv_cap;
-  const int32_t* gate;            // non-null: the general solver runs only while *gate != 0
+  int32_t *unit_off, *unit_np, *unit_fill, *unit_rows;   // G: per unit: piece list, pieces, fill cursor, rows
+  int32_t* unit_slot;             // G: multi-CTA units: first row slot
+  int4* msync;                    // 2 x kMaxGrid: barrier words of the multi-CTA class
+  int32_t *unit_pieces, *unit_pblk, *unit_prow, *unit_pbase;   // G: piece lists: id, block, rows, first row
+  int32_t* cls_list;              // kLists x cls_cap: units of each size class
+  int64_t cls_cap;
+  int32_t* clean_list;            // G: pieces of the step solved with their inverse
+  int32_t* clean_blk;             // G: their blocks
+  int32_t* wfast;                 // [kWSlots + 64] counters and cursors, then the labelling rounds' flags
+  int32_t* rowof;                 // P: row of a unique pair inside its component
+  int32_t* mrow;                  // Q: the same per member occurrence
+  float2* ent;                    // 4N: matrix entries (sqrt w, column) by slice, padding included
+  // row slots of the multi-CTA class
+  int32_t *rs_u, *rs_m, *rs_pm, *rs_len;
+  int4* rs_slice;                 // per slice: where its entries are
+  float *rs_y, *rs_r, *rs_p, *rs_ap, *rs_dz, *rs_di, *rs_zh, *rs_zl;
   float4* samples;
   float4* mom1;      // Adam first moment (M), null otherwise
   float4* mom2;      // pSGLD / Adam second moment (M), null for SGLD
@@ -240,21 +205,36 @@ struct StepView {
 };
 
 constexpr int kMaxGrid = 4096;
-// wfast[] slots of the piece-inverse whitening
+// size classes of the components solved by conjugate gradients: one warp, CTAs of
+// 8, 16 and 32 warps, several CTAs; the late list holds pieces whose stored
+// inverse did not converge
 enum : int {
-  kWUnits = 0, kWCursor = 1, kWGeneral = 2, kWRounds = 3,
-  kWBigS = 4,      // units solved by the second pass (large shared-node sets)
-  kWCycSm = 5,     // SM cycles / 1024 spent on units of the first pass
-  kWCycBig = 6,    // the same for the second pass
-  kWDefer = 7,     // units deferred to the second pass
-  kWCursor2 = 8,   // work cursor of the second pass
-  kWClean = 9,     // single pieces of the step (no shared node)
-  kWCursorC = 10,  // work cursor of the single-piece solver
-  // slots 11 and 13: unused
-  kWDefer2 = 12,   // units deferred from the CTA pass to the last pass
-  kWCursorS = 14,  // work cursor of the CTA inverse of the largest S
-  kWCursorS2 = 15, // work cursor of the register inverse of S at 97..128 shared nodes
-  kWSlots = 16
+  kClsWarp = 0, kClsSmall = 1, kClsMid = 2, kClsCta = 3, kClsMulti = 4, kClasses = 5, kClsLate = 5, kLists = 6
+};
+constexpr int kWarpRows = 64, kSmallRows = 256, kMidRows = 512, kCtaRows = 1024;
+constexpr int kWarpPieces = 32, kSmallPieces = 256, kMidPieces = 512, kCtaPieces = 1024;
+// Lines between the classes: the rows that 1 warp (two per lane), 8, 16 and 32
+// warps (one per lane) hold in registers, and the pieces whose tables fit beside
+// them in shared memory.
+__host__ __device__ constexpr int solve_class(int rows, int pieces) {
+  return rows <= kWarpRows && pieces <= kWarpPieces     ? kClsWarp
+         : rows <= kSmallRows && pieces <= kSmallPieces ? kClsSmall
+         : rows <= kMidRows && pieces <= kMidPieces     ? kClsMid
+         : rows <= kCtaRows && pieces <= kCtaPieces     ? kClsCta
+                                                        : kClsMulti;
+}
+// wfast[] slots
+enum : int {
+  kWUnits = 0,      // components solved by conjugate gradients
+  kWPieces = 1,     // their pieces
+  kWGeneral = 2,    // 1: a component needed several CTAs, or a stored inverse did not converge
+  kWClean = 3,      // pieces solved with their stored inverse
+  kWCursorC = 4,    // their work cursor
+  kWRowSlots = 5,   // row slots taken by the multi-CTA class
+  kWEntries = 6,    // entries taken from the pool
+  kWClass0 = 8,     // units per class list
+  kWCursor0 = 16,   // work cursors of the class lists
+  kWSlots = 24
 };
 constexpr int kCenChunk = 4096;   // events per centroid partial sum
 
