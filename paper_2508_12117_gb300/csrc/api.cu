@@ -175,17 +175,22 @@ cudaError_t upload_net(const spider_net* in, int precision, NetView* nv, std::ve
     n.W1 = p;
     if ((e = dupload(list, &p, in->b[0], (size_t)H, st))) return e;
     n.b1 = p;
-    std::vector<float> t((size_t)H * H);
+    const size_t HH = (size_t)H * H;
+    std::vector<float> t(precision == SPIDER_FP32 ? 6 * HH : 0);
     for (int l = 0; l < 3; ++l) {
       const float* W = in->W[l + 1];
-      for (int o = 0; o < H; ++o)
-        for (int i = 0; i < H; ++i) t[(size_t)i * H + o] = W[(size_t)o * H + i];
-      if ((e = dupload(list, &p, t.data(), t.size(), st))) return e;
-      n.Wt[l] = p;
-      if ((e = dupload(list, &p, W, (size_t)H * H, st))) return e;
-      n.Wn[l] = p;
+      if (precision == SPIDER_FP32) {
+        float* f = t.data() + l * HH;
+        for (int o = 0; o < H; ++o)
+          for (int i = 0; i < H; ++i) f[(size_t)i * H + o] = W[(size_t)o * H + i];
+        std::copy(W, W + HH, t.data() + (5 - l) * HH);
+      }
       if ((e = dupload(list, &p, in->b[l + 1], (size_t)H, st))) return e;
       n.bh[l] = p;
+    }
+    if (precision == SPIDER_FP32) {
+      if ((e = dupload(list, &p, t.data(), t.size(), st))) return e;
+      n.Wd = p;
     }
     if ((e = dupload(list, &p, in->W[4], (size_t)H, st))) return e;
     n.W5 = p;
@@ -200,7 +205,7 @@ cudaError_t upload_net(const spider_net* in, int precision, NetView* nv, std::ve
       n.tc = img;
       n.tc_scale = sc;
     }
-    // the transposed copy above must outlive the async copy
+    // the host copy above must outlive the async copy
     if ((e = cudaStreamSynchronize(st))) return e;
   }
   *nv = n;

@@ -119,20 +119,20 @@ extern "C" int spider_tt_pairs_noalloc(const spider_net* net, int64_t P, const f
   const size_t HH = (size_t)H * H;
   float* W1 = base;
   float* b1 = W1 + (size_t)H * 6;
-  float* Wn = b1 + H;          // 3 x H x H, (out, in)
-  float* Wt = Wn + 3 * HH;     // 3 x H x H, (in, out)
-  float* bh = Wt + 3 * HH;     // 3 x H
+  float* Wd = b1 + H;          // 6 x H x H: W2^T, W3^T, W4^T (in, out), W4, W3, W2 (out, in)
+  float* bh = Wd + 6 * HH;     // 3 x H
   float* W5 = bh + 3 * H;      // H
   float* slots = base + kNaWeights;
   float2* stage = reinterpret_cast<float2*>(slots + kNaSlots);
   e = cudaMemcpyAsync(W1, net->W[0], (size_t)H * 6 * sizeof(float), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b1, net->b[0], H * sizeof(float), cudaMemcpyHostToDevice, st);
   for (int l = 0; l < 3 && e == cudaSuccess; ++l) {
-    e = cudaMemcpyAsync(Wn + l * HH, net->W[l + 1], HH * sizeof(float), cudaMemcpyHostToDevice, st);
+    float* rev = Wd + (5 - l) * HH;
+    e = cudaMemcpyAsync(rev, net->W[l + 1], HH * sizeof(float), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(bh + l * H, net->b[l + 1], H * sizeof(float), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) {
-      k_transpose<<<(unsigned)((HH + 255) / 256), 256, 0, st>>>(Wn + l * HH, Wt + l * HH, H);
+      k_transpose<<<(unsigned)((HH + 255) / 256), 256, 0, st>>>(rev, Wd + l * HH, H);
       e = cudaGetLastError();
     }
   }
@@ -144,11 +144,8 @@ extern "C" int spider_tt_pairs_noalloc(const spider_net* net, int64_t P, const f
     nv.precision = SPIDER_FP32;
     nv.W1 = W1;
     nv.b1 = b1;
-    for (int l = 0; l < 3; ++l) {
-      nv.Wn[l] = Wn + l * HH;
-      nv.Wt[l] = Wt + l * HH;
-      nv.bh[l] = bh + l * H;
-    }
+    nv.Wd = Wd;
+    for (int l = 0; l < 3; ++l) nv.bh[l] = bh + l * H;
     nv.W5 = W5;
     nv.b5 = net->b[4][0];
     PairSource ps{};
@@ -156,8 +153,9 @@ extern "C" int spider_tt_pairs_noalloc(const spider_net* net, int64_t P, const f
     ps.rcv = reinterpret_cast<const float4*>(rcv);
     ps.n_host = P;
     TTOut o{stage, reinterpret_cast<float4*>(J)};
-    // launch_tt sizes the FP32 MLP grid as 2 x (its SM argument): kNaCtas CTAs,
-    // one scratch slot each
+    // launch_tt sizes the FP32 MLP grid as 2 x (its SM argument) CTAs at H = 256,
+    // kNaCtas, one scratch slot each; narrower networks take more CTAs with
+    // slots that much smaller
     e = launch_tt(nv, ps, o, kNaCtas / 2, slots, st, 2);
   }
   if (e == cudaSuccess)

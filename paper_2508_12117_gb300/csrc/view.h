@@ -28,8 +28,9 @@ struct NetView {
   float inv_v_hi, inv_v_lo;   // 1/v0 as a double-float
   const float* W1;   // H x 6 (out, in)
   const float* b1;   // H
-  const float* Wt[3];  // W2..W4 transposed: [in][out] (forward operand)
-  const float* Wn[3];  // W2..W4 as given: [out][in] (backward operand)
+  // FP32: the six products' weights in the order the kernel reads them:
+  // W2^T, W3^T, W4^T ([in][out], forward), W4, W3, W2 ([out][in], reverse)
+  const float* Wd;
   const float* bh[3];  // b2..b4
   const float* W5;     // H
   float b5;
