@@ -48,6 +48,13 @@ struct spider_ctx {
   uint64_t wait_ns = 2000000000ull; // limit of the bounded device-side waits
   double* state_dev = nullptr;     // M x 4 FP64 read-back buffer (caller order)
   float4* grad_dev = nullptr;      // M gradient read-back buffer (caller order)
+  // made by the first call that needs them: the observation filters' mask, their
+  // scratch and the caller's index of each observation (null where the orders
+  // are the same), the posterior summaries' truth and results
+  uint8_t* mask_dev = nullptr;
+  uint8_t* mask_scratch = nullptr;
+  int32_t* ord_dev = nullptr;
+  double* uq_dev = nullptr;
   int grid_ev = 1;                 // CTAs of the read-back kernels
   // stage events of a timed evaluation: start, after selection + pair table,
   // travel times, k_resid, k_merge_rhs, whitening, k_final, k_merge_s,
@@ -259,7 +266,7 @@ cudaError_t step_sequence(spider_ctx* c, int64_t n_b, bool logpost, bool timed) 
   src.sta_lo = v.sta_lo;
   src.n_dev = v.counters + kCntPairs;
   src.n_host = v.P;
-  TTOut out{v.T2, v.J};
+  TTOut out{v.T2, v.J, nullptr, nullptr};
   TRY(launch_tt(c->net, src, out, c->num_sms, c->tt_scratch, st, c->knobs[2]));
   if (timed) TRY(cudaEventRecord(c->ev[2], st));
   TRY(launch_resid(v, n_b, c->gu, st, timed ? &c->ev[3] : nullptr, 256 * c->knobs[5]));
@@ -353,6 +360,26 @@ int evaluate(spider_ctx* c, uint64_t seed, int mode, float eps) {
 }
 
 }  // namespace
+
+// The observation filters' device buffers (the mask is written in the caller's
+// order on the device: one copy instead of a pass over N on the host).
+static int mask_buffers(spider_ctx* c, size_t scratch) {
+  if (c->mask_dev) return SPIDER_OK;
+  const size_t N = c->v.N;
+  bool same = true;
+  for (size_t n = 0; n < N && same; ++n) same = c->ord[n] == (int32_t)n;
+  uint8_t *m = nullptr, *sc = nullptr;
+  int32_t* o = nullptr;
+  cudaError_t e = dalloc(c->allocs, &sc, scratch);
+  if (e == cudaSuccess && !same) e = dupload(c->allocs, &o, c->ord.data(), N, c->stream);
+  if (e == cudaSuccess) e = dalloc(c->allocs, &m, N);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+  if (e != cudaSuccess) return cuda_fail(c, e, "filter buffers");
+  c->mask_scratch = sc;
+  c->ord_dev = o;
+  c->mask_dev = m;
+  return SPIDER_OK;
+}
 
 void spider::set_static_error(const char* msg) { g_static_err = msg; }
 
@@ -972,63 +999,49 @@ int spider_set_moments(spider_ctx* c, const double* m, const double* v) {
 int spider_outlier_mask(spider_ctx* c, double k_mad, uint8_t* keep_out, int64_t* n_kept_out, double* med_out,
                         double* mad_out) {
   if (!c || !(k_mad > 0.0) || !std::isfinite(k_mad)) return SPIDER_E_INVAL;
-  int rc = evaluate(c, 0, 0, 0.f);          // full-batch residuals at the current state
+  int rc = mask_buffers(c, outlier_scratch_bytes(c->n_sub));
   if (rc) return rc;
-  rc = spider_sync(c);
+  rc = evaluate(c, 0, 0, 0.f);              // full-batch residuals at the current state
   if (rc) return rc;
   const int ns = c->n_sub;
-  const size_t N = c->v.N;
-  void* scratch = nullptr;
-  uint8_t* keep = nullptr;
-  CK(c, cudaMallocAsync(&scratch, outlier_scratch_bytes(ns), c->stream));
-  cudaError_t e = cudaMallocAsync(&keep, N > 0 ? N : 1, c->stream);
   std::vector<float> med(ns), mad(ns);
   int64_t kept = 0;
-  if (e == cudaSuccess)
-    e = launch_outlier(c->v, ns, (float)k_mad, scratch, keep, c->num_sms, c->stream, med.data(), mad.data(), &kept);
-  std::vector<uint8_t> hk;
-  if (e == cudaSuccess && keep_out) {
-    hk.resize(N);
-    e = cudaMemcpyAsync(hk.data(), keep, N, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  }
-  if (keep) cudaFreeAsync(keep, c->stream);
-  cudaFreeAsync(scratch, c->stream);
+  const cudaError_t e = launch_outlier(c->v, ns, (float)k_mad, c->mask_scratch, c->ord_dev, c->mask_dev, c->num_sms,
+                                       c->stream, med.data(), mad.data(), &kept);
   if (e != cudaSuccess) return cuda_fail(c, e, "outlier mask");
-  if (keep_out)
-    for (size_t n = 0; n < N; ++n) keep_out[c->ord[n]] = hk[n];
+  rc = check_device_error(c);
+  if (rc) return rc;
+  if (keep_out) {
+    CK(c, cudaMemcpyAsync(keep_out, c->mask_dev, c->v.N, cudaMemcpyDeviceToHost, c->stream));
+    CK(c, cudaStreamSynchronize(c->stream));
+  }
   if (n_kept_out) *n_kept_out = kept;
   for (int i = 0; i < ns; ++i) {
     if (med_out) med_out[i] = med[i];
     if (mad_out) mad_out[i] = mad[i];
   }
-  return check_device_error(c);
+  return SPIDER_OK;
 }
 
 int spider_linearisation_mask(spider_ctx* c, double max_rel, uint8_t* keep_out, int64_t* n_kept_out) {
   if (!c || !(max_rel >= 0.0) || !std::isfinite(max_rel)) return SPIDER_E_INVAL;
-  int rc = evaluate(c, 0, 0, 0.f);          // T and dT/dx of every pair at the current state
+  int rc = mask_buffers(c, outlier_scratch_bytes(c->n_sub));
   if (rc) return rc;
-  rc = spider_sync(c);
+  rc = evaluate(c, 0, 0, 0.f);              // T and dT/dx of every pair at the current state
   if (rc) return rc;
-  const size_t N = c->v.N;
-  uint8_t* keep = nullptr;
-  unsigned long long* kept = nullptr;
-  CK(c, cudaMallocAsync(&kept, sizeof(unsigned long long), c->stream));
-  cudaError_t e = cudaMallocAsync(&keep, N > 0 ? N : 1, c->stream);
-  if (e == cudaSuccess) e = launch_linfilter(c->v, c->nb_full, (float)max_rel, keep, kept, c->stream);
-  std::vector<uint8_t> hk(keep_out ? N : 0);
+  unsigned long long* kept = reinterpret_cast<unsigned long long*>(c->mask_scratch);
+  cudaError_t e = launch_linfilter(c->v, c->nb_full, (float)max_rel, c->ord_dev, c->mask_dev, kept, c->stream);
   unsigned long long kh = 0;
-  if (e == cudaSuccess && keep_out) e = cudaMemcpyAsync(hk.data(), keep, N, cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&kh, kept, sizeof(kh), cudaMemcpyDeviceToHost, c->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  if (keep) cudaFreeAsync(keep, c->stream);
-  cudaFreeAsync(kept, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "linearisation mask");
-  if (keep_out)
-    for (size_t n = 0; n < N; ++n) keep_out[c->ord[n]] = hk[n];
+  rc = check_device_error(c);
+  if (rc) return rc;
+  if (keep_out) {
+    CK(c, cudaMemcpyAsync(keep_out, c->mask_dev, c->v.N, cudaMemcpyDeviceToHost, c->stream));
+    CK(c, cudaStreamSynchronize(c->stream));
+  }
   if (n_kept_out) *n_kept_out = (int64_t)kh;
-  return check_device_error(c);
+  return SPIDER_OK;
 }
 
 int spider_uq(spider_ctx* c, const double* truth, double lo_pct, double hi_pct, double* median_out,
@@ -1044,38 +1057,26 @@ int spider_uq(spider_ctx* c, const double* truth, double lo_pct, double hi_pct, 
   }
   const int64_t first = c->n_samples - have;
   const size_t M = c->v.M;
-  std::vector<double> toff;
-  if (truth) {
-    toff.resize(4 * M);
-    for (size_t m = 0; m < M; ++m)
-      for (int a = 0; a < 4; ++a) toff[4 * m + a] = truth[4 * (size_t)c->ev_old[m] + a] - c->th0[4 * m + a];
+  // truth and the four results, kept for the next call
+  if (!c->uq_dev) {
+    double* p = nullptr;
+    const cudaError_t ea = dalloc(c->allocs, &p, 5 * 4 * M);
+    if (ea != cudaSuccess) return cuda_fail(c, ea, "summary buffers");
+    c->uq_dev = p;
   }
-  double* d = nullptr;
+  double* const d = c->uq_dev;
   const size_t nb = 4 * M * sizeof(double);
-  CK(c, cudaMallocAsync(&d, 5 * nb, c->stream));
-  double* dt = d;
-  double* outs[4] = {d + 4 * M, d + 8 * M, d + 12 * M, d + 16 * M};
-  double* want[4] = {median_out, halfwidth_out, calib_out, ess_out};
+  double* want[4] = {median_out, halfwidth_out, truth ? calib_out : nullptr, ess_out};
+  double* dev[4];
+  for (int k = 0; k < 4; ++k) dev[k] = want[k] ? d + (1 + k) * 4 * M : nullptr;
   cudaError_t e = cudaSuccess;
-  if (truth) e = cudaMemcpyAsync(dt, toff.data(), nb, cudaMemcpyHostToDevice, c->stream);
+  if (truth) e = cudaMemcpyAsync(d, truth, nb, cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess)
-    e = launch_uq(c->v, first % c->v.sample_cap, (int)have, truth ? dt : nullptr, lo_pct, hi_pct,
-                  want[0] ? outs[0] : nullptr, want[1] ? outs[1] : nullptr, truth && want[2] ? outs[2] : nullptr,
-                  want[3] ? outs[3] : nullptr, c->stream);
-  std::vector<double> h(4 * M);
-  for (int k = 0; k < 4 && e == cudaSuccess; ++k) {
-    if (!want[k] || (k == 2 && !truth)) continue;
-    e = cudaMemcpyAsync(h.data(), outs[k], nb, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    if (e != cudaSuccess) break;
-    for (size_t m = 0; m < M; ++m)
-      for (int a = 0; a < 4; ++a) {
-        double val = h[4 * m + a];
-        if (k == 0) val += c->th0[4 * m + a];          // the median back to absolute coordinates
-        want[k][4 * (size_t)c->ev_old[m] + a] = val;
-      }
-  }
-  cudaFreeAsync(d, c->stream);
+    e = launch_uq(c->v, first % c->v.sample_cap, (int)have, truth ? d : nullptr, lo_pct, hi_pct, dev[0], dev[1], dev[2],
+                  dev[3], c->stream);
+  for (int k = 0; k < 4 && e == cudaSuccess; ++k)
+    if (want[k]) e = cudaMemcpyAsync(want[k], dev[k], nb, cudaMemcpyDeviceToHost, c->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "posterior summaries");
   if (calib_out && !truth)
     for (size_t i = 0; i < 4 * M; ++i) calib_out[i] = std::nan("");
@@ -1327,27 +1328,14 @@ int spider_tt_pairs(const spider_netdev* nd, int64_t P, const float* src, const 
   if (P == 0) return SPIDER_OK;
   if (P > (int64_t)INT32_MAX) return SPIDER_E_INVAL;
   cudaStream_t st = (cudaStream_t)stream;
-  // T is produced as (hi, lo) pairs; split into the caller's arrays afterwards
-  float2* T2 = nullptr;
-  cudaError_t e = cudaMallocAsync(&T2, (size_t)P * sizeof(float2), st);
-  if (e != cudaSuccess) { g_static_err = cudaGetErrorString(e); return SPIDER_E_OOM; }
   PairSource ps{};
   ps.src = reinterpret_cast<const float4*>(src);
   ps.rcv = reinterpret_cast<const float4*>(rcv);
   ps.n_host = P;
-  TTOut o{T2, reinterpret_cast<float4*>(J)};
-  e = launch_tt(nd->net, ps, o, nd->num_sms, nd->scratch, st, 2);
-  if (e == cudaSuccess)
-    e = cudaMemcpy2DAsync(T_hi, sizeof(float), T2, sizeof(float2), sizeof(float), (size_t)P,
-                          cudaMemcpyDeviceToDevice, st);
-  if (e == cudaSuccess && T_lo)
-    e = cudaMemcpy2DAsync(T_lo, sizeof(float), reinterpret_cast<float*>(T2) + 1, sizeof(float2), sizeof(float),
-                          (size_t)P, cudaMemcpyDeviceToDevice, st);
-  cudaError_t e2 = cudaFreeAsync(T2, st);
-  if (e == cudaSuccess) e = e2;
+  cudaError_t e = launch_times(nd->net, ps, T_hi, T_lo, J, nullptr, nd->num_sms, nd->scratch, st);
   if (e != cudaSuccess) {
     g_static_err = cudaGetErrorString(e);
-    return SPIDER_E_CUDA;
+    return e == cudaErrorMemoryAllocation ? SPIDER_E_OOM : SPIDER_E_CUDA;
   }
   return SPIDER_OK;
 }

@@ -785,7 +785,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         df32 d[3];
         const df32 rr = geometry(pg, d);
         const df32 T = df_add_f(df_mul_f(rr, net.b5), rr.hi * dtau);
-        out.T2[u] = make_float2(T.hi, T.lo);
+        store_time(out, u, T.hi, T.lo);
         if (out.J) {
           const float tau = net.b5 + dtau;
           const float f = tau / rr.hi;

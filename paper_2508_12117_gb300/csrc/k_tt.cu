@@ -12,6 +12,8 @@
 //    This file holds the FP32 SIMT form; the tensor-core forms live in k_mlp_tc.cu.
 #include <cuda_runtime.h>
 
+#include <cstdint>
+
 #include "dfloat.cuh"
 #include "kernels.h"
 #include "pairs.cuh"
@@ -31,7 +33,7 @@ __global__ void k_tt_homogeneous(NetView net, PairSource src, TTOut out) {
     df32 d[3];
     const df32 r = geometry(g, d);
     const df32 T = df_mul(r, inv_v);
-    out.T2[u] = make_float2(T.hi, T.lo);
+    store_time(out, u, T.hi, T.lo);
     if (out.J) {
       const float f = net.inv_v_hi / r.hi;
       out.J[u] = make_float4(d[0].hi * f, d[1].hi * f, d[2].hi * f, 0.f);
@@ -54,7 +56,7 @@ __global__ void k_tt_gradient(NetView net, PairSource src, TTOut out) {
     const float X = gg * gg * r.hi * r.hi / (2.f * vs * vr);
     const float sq = sqrtf(X * (2.f + X));
     const float T = log1pf(X + sq) / gg;
-    out.T2[u] = make_float2(T, 0.f);
+    store_time(out, u, T, 0.f);
     if (out.J) {
       const float dTdX = 1.f / (gg * sq);
       const float c = dTdX * gg * gg / (vs * vr);
@@ -376,7 +378,7 @@ __global__ void __launch_bounds__(Mlp32<H, WIDE>::kThreads, Mlp32<H, WIDE>::kCta
       const df32 r = geometry(g, d);
       // T = r * (b5 + dtau): the bias part in double-float, the network part in FP32
       const df32 T = df_add_f(df_mul_f(r, net.b5), r.hi * s[0]);
-      out.T2[u] = make_float2(T.hi, T.lo);
+      store_time(out, u, T.hi, T.lo);
       if (out.J) {
         const float tau = net.b5 + s[0];
         const float f = tau / r.hi;
@@ -440,6 +442,34 @@ cudaError_t launch_tt(const NetView& net, const PairSource& src, TTOut out, int 
     case 256: return launch_mlp_fp32<256>(net, src, out, num_sms, ctas_per_sm, scratch, st);
     default: return cudaErrorNotSupported;
   }
+}
+
+cudaError_t launch_times(const NetView& net, const PairSource& src, float* T_hi, float* T_lo, float* J, float2* stage,
+                         int num_sms, float* scratch, cudaStream_t st) {
+  const size_t P = (size_t)src.n_host;
+  auto apart = [](const void* a, size_t na, const void* b, size_t nb) {
+    const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+    return !a || !b || x + na <= y || y + nb <= x;
+  };
+  const void* other[3] = {src.src, src.rcv, J};
+  bool direct = true;
+  for (const void* o : other) direct = direct && apart(T_hi, 4 * P, o, 16 * P) && apart(T_lo, 4 * P, o, 16 * P);
+  direct = direct && apart(T_hi, 4 * P, T_lo, 4 * P);
+  if (direct) return launch_tt(net, src, TTOut{nullptr, reinterpret_cast<float4*>(J), T_hi, T_lo}, num_sms, scratch, st, 2);
+  float2* T2 = stage;
+  cudaError_t e = cudaSuccess;
+  if (!T2 && (e = cudaMallocAsync(&T2, P * sizeof(float2), st)) != cudaSuccess) return cudaErrorMemoryAllocation;
+  e = launch_tt(net, src, TTOut{T2, reinterpret_cast<float4*>(J), nullptr, nullptr}, num_sms, scratch, st, 2);
+  if (e == cudaSuccess)
+    e = cudaMemcpy2DAsync(T_hi, sizeof(float), T2, sizeof(float2), sizeof(float), P, cudaMemcpyDeviceToDevice, st);
+  if (e == cudaSuccess && T_lo)
+    e = cudaMemcpy2DAsync(T_lo, sizeof(float), reinterpret_cast<float*>(T2) + 1, sizeof(float2), sizeof(float), P,
+                          cudaMemcpyDeviceToDevice, st);
+  if (!stage) {
+    const cudaError_t e2 = cudaFreeAsync(T2, st);
+    if (e == cudaSuccess) e = e2;
+  }
+  return e;
 }
 
 }  // namespace spider

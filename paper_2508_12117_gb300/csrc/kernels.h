@@ -15,6 +15,14 @@ size_t tt_scratch_floats(const NetView& net, int num_sms);
 // ctas_per_sm (1 or 2) shapes the FP32 MLP grid; scratch holds 2 x num_sms slots
 cudaError_t launch_tt(const NetView& net, const PairSource& src, TTOut out, int num_sms, float* scratch,
                       cudaStream_t st, int ctas_per_sm);
+// The same for the caller's arrays (raw pairs): the kernels write T_hi and T_lo
+// themselves.  Splitting staged (hi, lo) pairs afterwards cost an allocation and
+// two strided copies (47 pairs: 200 us a call that is waited for, 1.57 M pairs:
+// 0.12 ms); it is left for times that overlap another array, where a pair's
+// result may not be written before every pair has been read.  stage: P float2 of
+// the caller's, or null to allocate them on the stream.
+cudaError_t launch_times(const NetView& net, const PairSource& src, float* T_hi, float* T_lo, float* J, float2* stage,
+                         int num_sms, float* scratch, cudaStream_t st);
 cudaError_t launch_mlp_tc(const NetView& net, const PairSource& src, TTOut out, int num_sms,
                           float* scratch, cudaStream_t st);
 bool mlp_tc_supported(int H, int precision);
@@ -70,13 +78,15 @@ cudaError_t launch_solve_class(const StepView& v, int cls, int max_it, float tol
 cudaError_t launch_solve_multi(const StepView& v, int max_it, float tol, int grid, cudaStream_t st);
 // stage-1 outlier mask (k_outlier.cu)
 size_t outlier_scratch_bytes(int n_sub);
-cudaError_t launch_outlier(const StepView& v, int n_sub, float kmad, void* scratch, uint8_t* keep,
+// ord (nullable: the same): the caller's index of each observation, the order of keep
+cudaError_t launch_outlier(const StepView& v, int n_sub, float kmad, void* scratch, const int32_t* ord, uint8_t* keep,
                            int num_sms, cudaStream_t st, float* med_host, float* mad_host, int64_t* n_kept);
-cudaError_t launch_linfilter(const StepView& v, int64_t n_b, float max_rel, uint8_t* keep,
+cudaError_t launch_linfilter(const StepView& v, int64_t n_b, float max_rel, const int32_t* ord, uint8_t* keep,
                              unsigned long long* kept, cudaStream_t st);
 // posterior summaries (k_uq.cu)
 int uq_max_samples();
-cudaError_t launch_uq(const StepView& v, int64_t first, int n, const double* truth_off, double lo_pct,
+// truth and results: M x 4 FP64 on the device, the caller's event order
+cudaError_t launch_uq(const StepView& v, int64_t first, int n, const double* truth, double lo_pct,
                       double hi_pct, double* med, double* half, double* calib, double* ess, cudaStream_t st);
 cudaError_t launch_philox_words(uint64_t seed, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
                                 int64_t n, uint32_t* out, cudaStream_t st);

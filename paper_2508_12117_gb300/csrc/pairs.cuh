@@ -34,6 +34,15 @@ __device__ __forceinline__ void load_pair(const PairSource& s, int64_t u, PairGe
   }
 }
 
+__device__ __forceinline__ void store_time(const TTOut& o, int64_t u, float hi, float lo) {
+  if (o.T2) {
+    o.T2[u] = make_float2(hi, lo);
+  } else {
+    o.hi[u] = hi;
+    if (o.lo) o.lo[u] = lo;
+  }
+}
+
 // source - receiver per axis and the distance, in double-float
 __device__ __forceinline__ df32 geometry(const PairGeo& g, df32 d[3]) {
 #pragma unroll

@@ -152,18 +152,11 @@ extern "C" int spider_tt_pairs_noalloc(const spider_net* net, int64_t P, const f
     ps.src = reinterpret_cast<const float4*>(src);
     ps.rcv = reinterpret_cast<const float4*>(rcv);
     ps.n_host = P;
-    TTOut o{stage, reinterpret_cast<float4*>(J)};
     // launch_tt sizes the FP32 MLP grid as 2 x (its SM argument) CTAs at H = 256,
     // kNaCtas, one scratch slot each; narrower networks take more CTAs with
     // slots that much smaller
-    e = launch_tt(nv, ps, o, kNaCtas / 2, slots, st, 2);
+    e = launch_times(nv, ps, T_hi, T_lo, J, stage, kNaCtas / 2, slots, st);
   }
-  if (e == cudaSuccess)
-    e = cudaMemcpy2DAsync(T_hi, sizeof(float), stage, sizeof(float2), sizeof(float), (size_t)P,
-                          cudaMemcpyDeviceToDevice, st);
-  if (e == cudaSuccess && T_lo)
-    e = cudaMemcpy2DAsync(T_lo, sizeof(float), reinterpret_cast<float*>(stage) + 1, sizeof(float2),
-                          sizeof(float), (size_t)P, cudaMemcpyDeviceToDevice, st);
   if (e != cudaSuccess) {
     na_error(cudaGetErrorString(e));
     return SPIDER_E_CUDA;

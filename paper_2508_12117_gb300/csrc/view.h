@@ -58,8 +58,10 @@ struct PairSource {
 };
 
 struct TTOut {
-  float2* T2;   // (T_hi, T_lo)
+  float2* T2;   // (T_hi, T_lo), or null: hi and lo (may be null) apart
   float4* J;    // (dT/dx, dT/dy, dT/dz, 0), may be null
+  float* hi;
+  float* lo;
 };
 
 // Per-step parameters, read by the kernels from device memory (the host
