@@ -323,8 +323,8 @@ class Context:
         mad = np.empty(ns, np.float64)
         _check(load_library().spider_outlier_mask(self.h, float(k_mad), _ptr(keep, C.c_uint8), C.byref(kept),
                                                   _ptr(med, C.c_double), _ptr(mad, C.c_double)), self.h)
-        assert int(keep.sum()) == kept.value
-        return keep.astype(bool), med, mad
+        assert np.count_nonzero(keep) == kept.value
+        return keep.view(bool), med, mad
 
     def spider_linearisation_mask(self, max_rel: float = 0.05):
         """Keep mask over the caller's observations (linearisation error <= max_rel)."""
@@ -332,8 +332,8 @@ class Context:
         kept = C.c_int64()
         _check(load_library().spider_linearisation_mask(self.h, float(max_rel), _ptr(keep, C.c_uint8),
                                                         C.byref(kept)), self.h)
-        assert int(keep.sum()) == kept.value
-        return keep.astype(bool)
+        assert np.count_nonzero(keep) == kept.value
+        return keep.view(bool)
 
     def spider_uq(self, truth=None, lo_pct: float = 0.5, hi_pct: float = 99.5):
         """Per event and coordinate: median, credible half-width, calibration

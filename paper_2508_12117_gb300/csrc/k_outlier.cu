@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <vector>
 
 #include "dfloat.cuh"
 #include "kernels.h"
@@ -61,11 +62,52 @@ __global__ void k_sel_init(StepView v, SelSub* s, int n_sub) {
   s[i].mad = 0.f;
 }
 
-// histogram of the next 8 key bits of the values matching each rank's prefix;
-// mode 0: keys of r, mode 1: keys of |r - median|
-__global__ void k_sel_hist(const float* __restrict__ r, int64_t N, const SelSub* s, int n_sub, int mode,
-                           uint32_t mask, int shift, uint32_t* hist) {
+// Control block after the sub-problems: kept observations, CTAs of the running
+// histogram that have finished.
+struct SelCtl {
+  unsigned long long kept;
+  unsigned int done;
+};
+
+// The bin of 256 counts that holds rank k (the last one if none does), and the
+// rank inside it; one warp, eight bins per lane.
+__device__ __forceinline__ int pick_bin(const uint32_t* cnt, int64_t& k, int lane) {
+  uint32_t c[8], t = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    c[i] = cnt[8 * lane + i];
+    t += c[i];
+  }
+  int64_t before = t;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t y = __shfl_up_sync(0xffffffffu, before, o);
+    if (lane >= o) before += y;
+  }
+  const unsigned has = __ballot_sync(0xffffffffu, k < before);   // inclusive sums ascend over the lanes
+  const int src = has ? __ffs(has) - 1 : 31;
+  int64_t left = k - (before - t);
+  int bin = 8 * lane;
+#pragma unroll
+  for (int i = 0; i < 7; ++i)
+    if (left >= (int64_t)c[i] && bin == 8 * lane + i) {
+      left -= c[i];
+      ++bin;
+    }
+  k = __shfl_sync(0xffffffffu, left, src);
+  return __shfl_sync(0xffffffffu, bin, src);
+}
+
+// Histogram of the next 8 key bits of the values matching each rank's prefix
+// (mode 0: keys of r, mode 1: keys of |r - median|); the CTA that finishes last
+// picks the bin holding each rank, extends the prefixes and, after the last
+// digit, sets the median or the MAD and the ranks of the next selection.  One
+// launch a digit: a launch of its own for the pick, its bins searched by one
+// thread, took as long as the histogram.
+__global__ void __launch_bounds__(256) k_sel_digit(const float* __restrict__ r, int64_t N, SelSub* s, SelCtl* ctl,
+                                                   int n_sub, int mode, uint32_t mask, int shift, uint32_t* hist) {
   __shared__ uint32_t sh[kSmemSubs * 2 * kBins];
+  __shared__ int last;
   const bool use_smem = n_sub <= kSmemSubs;
   if (use_smem) {
     for (int i = threadIdx.x; i < n_sub * 2 * kBins; i += blockDim.x) sh[i] = 0;
@@ -89,52 +131,47 @@ __global__ void k_sel_hist(const float* __restrict__ r, int64_t N, const SelSub*
     for (int i = threadIdx.x; i < n_sub * 2 * kBins; i += blockDim.x)
       if (sh[i]) atomicAdd(&hist[i], sh[i]);
   }
-}
-
-// one block per sub-problem: pick the bin holding each rank, extend its prefix
-__global__ void k_sel_pick(SelSub* s, int shift, uint32_t* hist) {
-  __shared__ uint32_t cnt[kBins];
-  const int sb = blockIdx.x;
-  // both ranks on one path (odd count): rank 1 was not histogrammed, it reuses rank 0's
-  const bool same = s[sb].k[1] == s[sb].k[0] && s[sb].prefix[1] == s[sb].prefix[0];
+  __threadfence();
   __syncthreads();
-  for (int l = 0; l < 2; ++l) {
-    const int src = (l == 1 && same) ? 0 : l;
-    uint32_t* h = hist + ((size_t)sb * 2 + src) * kBins;
-    for (int i = threadIdx.x; i < kBins; i += blockDim.x) cnt[i] = h[i];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int64_t k = s[sb].k[l];
-      int b = 0;
-      for (; b < kBins - 1; ++b) {
-        if (k < (int64_t)cnt[b]) break;
-        k -= cnt[b];
-      }
-      s[sb].k[l] = k;
-      s[sb].prefix[l] |= (uint32_t)b << shift;
+  if (threadIdx.x == 0) last = atomicAdd(&ctl->done, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const int lane = threadIdx.x & 31;
+  for (int sb = threadIdx.x >> 5; sb < n_sub; sb += blockDim.x >> 5) {
+    // both ranks on one path (odd count): rank 1 was not histogrammed, it reuses rank 0's
+    const bool same = s[sb].k[1] == s[sb].k[0] && s[sb].prefix[1] == s[sb].prefix[0];
+    int64_t k[2];
+    uint32_t prefix[2];
+    for (int l = 0; l < 2; ++l) {
+      k[l] = s[sb].k[l];
+      const int b = pick_bin(hist + ((size_t)sb * 2 + (l == 1 && same ? 0 : l)) * kBins, k[l], lane);
+      prefix[l] = s[sb].prefix[l] | (uint32_t)b << shift;
     }
-    __syncthreads();
+    __syncwarp();
+    if (lane == 0) {
+      if (shift > 0) {
+        for (int l = 0; l < 2; ++l) {
+          s[sb].k[l] = k[l];
+          s[sb].prefix[l] = prefix[l];
+        }
+      } else {
+        const int64_t n = s[sb].hi - s[sb].lo;
+        const float m = n > 0 ? 0.5f * (fkey_inv(prefix[0]) + fkey_inv(prefix[1])) : 0.f;
+        if (mode == 0) s[sb].med = m;
+        else s[sb].mad = m;
+        s[sb].k[0] = n > 0 ? (n - 1) / 2 : 0;
+        s[sb].k[1] = n > 0 ? n / 2 : 0;
+        s[sb].prefix[0] = s[sb].prefix[1] = 0;
+      }
+    }
+    for (int i = lane; i < 2 * kBins; i += 32) hist[(size_t)sb * 2 * kBins + i] = 0;
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < 2 * kBins; i += blockDim.x) hist[(size_t)sb * 2 * kBins + i] = 0;
-}
-
-__global__ void k_sel_done(SelSub* s, int n_sub, int mode) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n_sub) return;
-  const float a = fkey_inv(s[i].prefix[0]), b = fkey_inv(s[i].prefix[1]);
-  const float m = s[i].hi > s[i].lo ? 0.5f * (a + b) : 0.f;
-  if (mode == 0) s[i].med = m;
-  else s[i].mad = m;
-  // reset the ranks for the next selection
-  const int64_t n = s[i].hi - s[i].lo;
-  s[i].k[0] = n > 0 ? (n - 1) / 2 : 0;
-  s[i].k[1] = n > 0 ? n / 2 : 0;
-  s[i].prefix[0] = s[i].prefix[1] = 0;
+  if (threadIdx.x == 0) ctl->done = 0;
 }
 
 __global__ void k_keep(const float* __restrict__ r, int64_t N, const SelSub* s, int n_sub, float kmad,
-                       uint8_t* keep, unsigned long long* kept) {
+                       const int32_t* __restrict__ ord, uint8_t* keep, unsigned long long* kept) {
   __shared__ int cnt;
   if (threadIdx.x == 0) cnt = 0;
   __syncthreads();
@@ -142,7 +179,7 @@ __global__ void k_keep(const float* __restrict__ r, int64_t N, const SelSub* s, 
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < N; e += (int64_t)gridDim.x * blockDim.x) {
     const int sb = sub_of(s, n_sub, e);
     const uint8_t k = fabsf(r[e] - s[sb].med) <= kmad * s[sb].mad ? 1 : 0;
-    keep[e] = k;
+    keep[ord ? ord[e] : e] = k;
     mine += k;
   }
   atomicAdd(&cnt, mine);
@@ -153,42 +190,40 @@ __global__ void k_keep(const float* __restrict__ r, int64_t N, const SelSub* s, 
 }  // namespace
 
 size_t outlier_scratch_bytes(int n_sub) {
-  return (size_t)n_sub * sizeof(SelSub) + (size_t)n_sub * 2 * kBins * sizeof(uint32_t) + 64;
+  return (size_t)n_sub * sizeof(SelSub) + sizeof(SelCtl) + (size_t)n_sub * 2 * kBins * sizeof(uint32_t);
 }
 
 // residuals r (canonical order, the full catalog) -> keep mask, per-sub median
 // and MAD (host copies), kept count.  scratch: outlier_scratch_bytes(n_sub).
-cudaError_t launch_outlier(const StepView& v, int n_sub, float kmad, void* scratch, uint8_t* keep,
+cudaError_t launch_outlier(const StepView& v, int n_sub, float kmad, void* scratch, const int32_t* ord, uint8_t* keep,
                            int num_sms, cudaStream_t st, float* med_host, float* mad_host, int64_t* n_kept) {
   SelSub* s = reinterpret_cast<SelSub*>(scratch);
-  uint32_t* hist = reinterpret_cast<uint32_t*>(s + n_sub);
-  unsigned long long* kept = reinterpret_cast<unsigned long long*>(hist + (size_t)n_sub * 2 * kBins);
+  SelCtl* ctl = reinterpret_cast<SelCtl*>(s + n_sub);
+  uint32_t* hist = reinterpret_cast<uint32_t*>(ctl + 1);
   cudaError_t e;
-  if ((e = cudaMemsetAsync(hist, 0, (size_t)n_sub * 2 * kBins * sizeof(uint32_t) + sizeof(unsigned long long), st)))
-    return e;
-  const int gs = (n_sub + 127) / 128;
-  k_sel_init<<<gs, 128, 0, st>>>(v, s, n_sub);
+  if ((e = cudaMemsetAsync(ctl, 0, sizeof(SelCtl) + (size_t)n_sub * 2 * kBins * sizeof(uint32_t), st))) return e;
+  k_sel_init<<<(n_sub + 127) / 128, 128, 0, st>>>(v, s, n_sub);
   const int grid = 2 * num_sms;
   for (int mode = 0; mode < 2; ++mode) {
     uint32_t mask = 0;
     for (int pass = 0; pass < 4; ++pass) {
       const int shift = 24 - 8 * pass;
-      k_sel_hist<<<grid, 256, 0, st>>>(v.r_obs, v.N, s, n_sub, mode, mask, shift, hist);
-      k_sel_pick<<<n_sub, 256, 0, st>>>(s, shift, hist);
+      k_sel_digit<<<grid, 256, 0, st>>>(v.r_obs, v.N, s, ctl, n_sub, mode, mask, shift, hist);
       mask |= 0xFFu << shift;
     }
-    k_sel_done<<<gs, 128, 0, st>>>(s, n_sub, mode);
   }
-  k_keep<<<grid, 256, 0, st>>>(v.r_obs, v.N, s, n_sub, kmad, keep, kept);
+  k_keep<<<grid, 256, 0, st>>>(v.r_obs, v.N, s, n_sub, kmad, ord, keep, &ctl->kept);
   if ((e = cudaGetLastError())) return e;
-  for (int i = 0; i < n_sub; ++i) {
-    if ((e = cudaMemcpyAsync(&med_host[i], &s[i].med, sizeof(float), cudaMemcpyDeviceToHost, st))) return e;
-    if ((e = cudaMemcpyAsync(&mad_host[i], &s[i].mad, sizeof(float), cudaMemcpyDeviceToHost, st))) return e;
-  }
-  unsigned long long kh = 0;
-  if ((e = cudaMemcpyAsync(&kh, kept, sizeof(kh), cudaMemcpyDeviceToHost, st))) return e;
+  // the sub-problems and the control block lie side by side: one copy
+  std::vector<uint8_t> host((size_t)n_sub * sizeof(SelSub) + sizeof(SelCtl));
+  if ((e = cudaMemcpyAsync(host.data(), s, host.size(), cudaMemcpyDeviceToHost, st))) return e;
   if ((e = cudaStreamSynchronize(st))) return e;
-  *n_kept = (int64_t)kh;
+  const SelSub* hs = reinterpret_cast<const SelSub*>(host.data());
+  for (int i = 0; i < n_sub; ++i) {
+    med_host[i] = hs[i].med;
+    mad_host[i] = hs[i].mad;
+  }
+  *n_kept = (int64_t)reinterpret_cast<const SelCtl*>(hs + n_sub)->kept;
   return cudaSuccess;
 }
 
@@ -203,7 +238,8 @@ cudaError_t launch_outlier(const StepView& v, int n_sub, float kmad, void* scrat
 namespace spider {
 namespace {
 
-__global__ void k_linfilter(StepView v, float max_rel, uint8_t* keep, unsigned long long* kept) {
+__global__ void k_linfilter(StepView v, float max_rel, const int32_t* __restrict__ ord, uint8_t* keep,
+                            unsigned long long* kept) {
   __shared__ int cnt;
   if (threadIdx.x == 0) cnt = 0;
   __syncthreads();
@@ -229,7 +265,7 @@ __global__ void k_linfilter(StepView v, float max_rel, uint8_t* keep, unsigned l
     const float lin = fmaf(Ji.x, dx, fmaf(Ji.y, dy, Ji.z * dz));
     const float err = fabsf(df_add_f(dT, -lin).hi);
     const uint8_t k = err <= max_rel * fabsf(dT.hi) ? 1 : 0;
-    keep[e0 + e] = k;
+    keep[ord ? ord[e0 + e] : e0 + e] = k;
     mine += k;
   }
   atomicAdd(&cnt, mine);
@@ -240,11 +276,11 @@ __global__ void k_linfilter(StepView v, float max_rel, uint8_t* keep, unsigned l
 }  // namespace
 
 // after a full-batch evaluation (every block selected, T and J per unique pair)
-cudaError_t launch_linfilter(const StepView& v, int64_t n_b, float max_rel, uint8_t* keep,
+cudaError_t launch_linfilter(const StepView& v, int64_t n_b, float max_rel, const int32_t* ord, uint8_t* keep,
                              unsigned long long* kept, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(kept, 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
-  if (n_b > 0) k_linfilter<<<(unsigned)n_b, 256, 0, st>>>(v, max_rel, keep, kept);
+  if (n_b > 0) k_linfilter<<<(unsigned)n_b, 256, 0, st>>>(v, max_rel, ord, keep, kept);
   return cudaGetLastError();
 }
 

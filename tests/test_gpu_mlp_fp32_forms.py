@@ -43,3 +43,28 @@ def test_forms_agree_and_match_the_oracle(H):
         for a, b in zip(run(n), want):
             assert torch.equal(a, b[:n]), n
     nd.close()
+
+
+@pytest.mark.parametrize("kind,precision", [("homogeneous", "FP32"), ("mlp", "FP32"), ("mlp", "BF16")])
+def test_times_may_overlap_the_inputs(kind, precision):
+    """T_hi and T_lo written over the source positions (and over each other's
+    neighbour) are those of separate arrays: every pair is read before any time
+    that lies on an input is written."""
+    torch = pytest.importorskip("torch")
+    net = binding.Net(binding.TT_MLP, mlp=synth.mlp_weights(64, 5)) if kind == "mlp" else \
+        binding.Net(binding.TT_HOMOGENEOUS, v0=6.0)
+    nd = binding.NetDevice(net, precision=getattr(binding, precision))
+    n = 20_001
+    torch.manual_seed(1)
+    s4, r4 = torch.rand(n, 4, device="cuda") * 40, torch.rand(n, 4, device="cuda") * 40
+    hi, lo, J = torch.empty(n, device="cuda"), torch.empty(n, device="cuda"), torch.empty(n, 4, device="cuda")
+    nd.spider_tt_pairs(n, s4.data_ptr(), r4.data_ptr(), hi.data_ptr(), lo.data_ptr(), J.data_ptr())
+    only = torch.empty(n, device="cuda")
+    nd.spider_tt_pairs(n, s4.data_ptr(), r4.data_ptr(), only.data_ptr(), 0, 0)
+    s, J2 = s4.clone(), torch.empty(n, 4, device="cuda")
+    over = s.view(-1)
+    nd.spider_tt_pairs(n, s.data_ptr(), r4.data_ptr(), over.data_ptr(), over.data_ptr() + 4 * n, J2.data_ptr())
+    torch.cuda.synchronize()
+    assert torch.equal(only, hi)
+    assert torch.equal(over[:n], hi) and torch.equal(over[n:2 * n], lo) and torch.equal(J2, J)
+    nd.close()
