@@ -452,6 +452,14 @@ int build_whitening(spider_ctx* c, const Prep& P, bool want_inverses) {
   UPF(mem_rp, T.mem_rp.data(), Q + 1);
   UPF(edge_pos, T.edge_pos.data(), T.edge_pos.size());
   UPF(edge_sw, T.edge_sw.data(), T.edge_sw.size());
+  {
+    std::vector<int32_t> nm(Q);
+    for (int64_t b = 0; b < P.NB; ++b)
+      for (int32_t q = P.blk_node_off[b]; q < P.blk_node_off[b + 1]; ++q)
+        nm[q] = T.piece_node_off[T.blk_piece_off[b] + T.node_piece[q]] + T.node_ppos[q];
+    UPF(node_mem, nm.data(), Q);
+    if ((e = cudaStreamSynchronize(st))) return cuda_fail(c, e, "upload sync");
+  }
   ALF(owner_b, Q);
   ALF(plab, G); ALF(prow, G); ALF(pmulti, G); ALF(pcount, G); ALF(urows, G);
   ALF(unit_of, G); ALF(unit_off, G); ALF(unit_np, G); ALF(unit_fill, G); ALF(unit_rows, G);
@@ -472,7 +480,7 @@ int build_whitening(spider_ctx* c, const Prep& P, bool want_inverses) {
     // rows of the multi-CTA class in whole slices: such a unit has more than
     // kCtaRows rows, or more than kCtaPieces pieces
     const size_t cap = PP + PP / 32 + G / 32 + 64;
-    ALF(rs_u, cap); ALF(rs_m, cap); ALF(rs_pm, cap); ALF(rs_len, cap); ALF(rs_slice, cap / 32 + 1);
+    ALF(rs_u, cap); ALF(rs_m, cap); ALF(rs_q, cap); ALF(rs_len, cap); ALF(rs_slice, cap / 32 + 1);
     ALF(rs_y, cap); ALF(rs_r, cap); ALF(rs_p, cap); ALF(rs_ap, cap); ALF(rs_dz, cap); ALF(rs_di, cap);
     ALF(rs_zh, cap); ALF(rs_zl, cap);
   }
@@ -687,6 +695,7 @@ int create_impl(const spider_catalog* cat, const spider_stations* sta, const spi
   AL(sel, NB);
   AL(blk_stamp, NB);
   AL(owner_q, Q);
+  AL(next_q, Q);
   AL(multi, Q);
   AL(loc2u, Q);
   AL(blk_owner_cnt, NB);

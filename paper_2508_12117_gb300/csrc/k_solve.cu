@@ -40,17 +40,6 @@ constexpr float kAim = 1e-4f;
 constexpr int kMaxReplace = 8;       // replacements at most
 constexpr int kMultiThreads = 512;   // threads per CTA of the multi-CTA class
 
-struct Occurrence {
-  int32_t m, pm0;                    // member index and the first member of its piece
-};
-
-__device__ __forceinline__ Occurrence occurrence(const StepView& v, int32_t q, int32_t b) {
-  Occurrence o;
-  o.pm0 = v.piece_node_off[v.blk_piece_off[b] + v.node_piece[q]];
-  o.m = o.pm0 + v.node_ppos[q];
-  return o;
-}
-
 // Where the entries of a slice are.  Steps [0, ss) sit in shared memory from sb
 // on, 32 words a step (rows shorter than `steps` padded with zero weights, so
 // the loop needs no predicate); the other steps in the pool in global memory:
@@ -65,16 +54,13 @@ struct EntrySmem {
   uint16_t* col;
 };
 
-// entries of a row: its edges over all selected occurrences of the pair
-__device__ __forceinline__ int row_len(const StepView& v, int tag, int32_t u, int32_t m) {
-  if (!v.umulti[u]) return v.mem_rp[m + 1] - v.mem_rp[m];
-  const int32_t p = v.uniq_pair[u];
-  int len = 0;
-  for (int32_t i = v.inc_off[p], i1 = v.inc_off[p + 1]; i < i1; ++i) {
-    const int32_t b = v.inc_b[i];
-    if (v.blk_stamp[b] != tag) continue;
-    const Occurrence o = occurrence(v, v.inc_q[i], b);
-    len += v.mem_rp[o.m + 1] - v.mem_rp[o.m];
+// entries of a row: its edges over all selected occurrences of the pair, from
+// the owner (local node q, member m) on
+__device__ __forceinline__ int row_len(const StepView& v, int32_t q, int32_t m) {
+  int len = v.mem_rp[m + 1] - v.mem_rp[m];
+  for (q = v.next_q[q]; q >= 0; q = v.next_q[q]) {
+    m = v.node_mem[q];
+    len += v.mem_rp[m + 1] - v.mem_rp[m];
   }
   return len;
 }
@@ -85,17 +71,14 @@ __device__ __forceinline__ int slice_steps(int len) { return ((int)__reduce_max_
 // (lane = row of `len` entries, 0 where there is none), its first ss steps to
 // shared memory and the others to a range taken from the pool.  A row's entries
 // run over its occurrences in block order, then in observation order.
-__device__ __forceinline__ Slice fill_slice(const StepView& v, int tag, int lane, int len, int steps, int row,
-                                            int32_t u, int32_t m, int32_t pm0, EntrySmem es, int sb, int ss) {
+__device__ __forceinline__ Slice fill_slice(const StepView& v, int lane, int len, int steps, int row, int32_t q,
+                                            int32_t m, EntrySmem es, int sb, int ss) {
   const unsigned lt = (1u << lane) - 1u;
-  int32_t t = 0, e = 0, e1 = 0;
+  int32_t e = 0, e1 = 0, pm0 = 0;
   if (len > 0) {
-    if (!v.umulti[u]) {
-      e = v.mem_rp[m];
-      e1 = e + len;
-    } else {
-      t = v.inc_off[v.uniq_pair[u]];
-    }
+    e = v.mem_rp[m];
+    e1 = v.mem_rp[m + 1];
+    pm0 = m - v.node_ppos[q];
   }
   Slice s{sb, ss, 0, len, steps};
   const int rest = __reduce_add_sync(0xffffffffu, len > ss ? len - ss : 0);
@@ -122,15 +105,12 @@ __device__ __forceinline__ Slice fill_slice(const StepView& v, int tag, int lane
       ei[i] = 0;
       pm[i] = 0;
       if (j + i < len) {
-        while (e == e1) {              // the next selected occurrence (multi rows)
-          const int32_t b = v.inc_b[t];
-          if (v.blk_stamp[b] == tag) {
-            const Occurrence o = occurrence(v, v.inc_q[t], b);
-            pm0 = o.pm0;
-            e = v.mem_rp[o.m];
-            e1 = v.mem_rp[o.m + 1];
-          }
-          ++t;
+        while (e == e1) {              // the next selected occurrence
+          q = v.next_q[q];
+          m = v.node_mem[q];
+          e = v.mem_rp[m];
+          e1 = v.mem_rp[m + 1];
+          pm0 = m - v.node_ppos[q];
         }
         ei[i] = e++;
         pm[i] = pm0;
@@ -211,37 +191,45 @@ __device__ __forceinline__ float slice_mul(const float2* ent, EntrySmem es, cons
   return s;
 }
 
-// the same in double-float
+// the same in double-float; even and odd steps in two sums, so that one chain of
+// additions does not bound it
 __device__ __forceinline__ df32 slice_mul_df(const float2* ent, EntrySmem es, const Slice& sl, int lane, df32 zr,
                                              const float* zh, const float* zl) {
-  df32 acc = {0.f, 0.f};
+  df32 acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
+  auto term = [&](float w, int c) {
+    return df_mul(df_two_prod(w, w), df_add(zr, df32{-zh[c], -zl[c]}));
+  };
+  const float* ws = es.sw + sl.sb + lane;
+  const uint16_t* cs = es.col + sl.sb + lane;
+  for (int j = 0; j < sl.ss; j += 4, ws += 4 * 32, cs += 4 * 32) {
+    df32 t[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) t[i] = term(ws[32 * i], cs[32 * i]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i & 1] = df_add(acc[i & 1], t[i]);
+  }
   const unsigned lt = (1u << lane) - 1u;
   int at = sl.gb >= 0 ? sl.gb + lane : ~sl.gb;
-#pragma unroll 4
-  for (int j = 0; j < sl.steps; ++j) {
-    float w = 0.f;
-    int c = 0;
-    if (j < sl.ss) {
-      w = es.sw[sl.sb + 32 * j + lane];
-      c = es.col[sl.sb + 32 * j + lane];
-    } else {
-      int i = at;
+  for (int j = sl.ss; j < sl.steps; j += 4) {
+    float2 x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      int k = at;
       if (sl.gb >= 0) {
         at += 32;
       } else {
-        const unsigned mask = __ballot_sync(0xffffffffu, j < sl.len);
-        i = at + __popc(mask & lt);
+        const unsigned mask = __ballot_sync(0xffffffffu, j + i < sl.len);
+        k = at + __popc(mask & lt);
         at += __popc(mask);
       }
-      if (j < sl.len) {
-        const float2 x = ent[i];
-        w = x.x;
-        c = __float_as_int(x.y);
-      }
+      x[i] = make_float2(0.f, 0.f);
+      if (j + i < sl.len) x[i] = ent[k];
     }
-    if (j < sl.len) acc = df_add(acc, df_mul(df_two_prod(w, w), df_add(zr, df32{-zh[c], -zl[c]})));
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (j + i < sl.len) acc[i & 1] = df_add(acc[i & 1], term(x[i].x, __float_as_int(x[i].y)));
   }
-  return acc;
+  return df_add(acc[0], acc[1]);
 }
 
 // u - lambda z - B^T B z of one row, rounded to FP32
@@ -298,7 +286,7 @@ struct SolveSmem {
   static constexpr int R = NW * RPT * 32;
   union {
     struct {
-      int32_t u[R], m[R], pm0[R], len[R];   // set-up: unique pair, member, its piece's first member
+      int32_t u[R], m[R], q[R], len[R];     // set-up: unique pair, member, local node, entries
     } row;
     struct {
       float y[R], zh[R], zl[R];
@@ -365,7 +353,6 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS) k_solve(StepView v, int cls,
   const int tid = threadIdx.x % (NW * 32), w = tid >> 5, lane = tid & 31;
   constexpr int NT = NW * 32;
   const unsigned lt = (1u << lane) - 1u;
-  const int tag = v.prm->tag;
   const float lam = v.lam;
   const int32_t count = v.wfast[kWClass0 + cls];
   const int32_t* list = v.cls_list + (int64_t)cls * v.cls_cap;
@@ -408,7 +395,7 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS) k_solve(StepView v, int cls,
           const int32_t u = v.loc2u[q];
           S.row.u[row] = u;
           S.row.m[row] = m;
-          S.row.pm0[row] = pm0;
+          S.row.q[row] = q;
         }
         row0 += __popc(mask);
       }
@@ -418,7 +405,7 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS) k_solve(StepView v, int cls,
     // numbers of steps: the lengths of a minibatch run from 1 to 24 around a mean
     // of 6, and in member order every slice ran to its longest
     {
-      int32_t u[RPT], m[RPT], pm0[RPT];
+      int32_t u[RPT], m[RPT], q[RPT];
       int len[RPT], bin[RPT], rank[RPT];
       for (int i = tid; i < kLenBins * NW * RPT; i += NT) S.bin[i] = 0;
       group_sync<NW>();
@@ -429,8 +416,8 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS) k_solve(StepView v, int cls,
         if (row < rows) {
           u[k] = S.row.u[row];
           m[k] = S.row.m[row];
-          pm0[k] = S.row.pm0[row];
-          len[k] = row_len(v, tag, u[k], m[k]);
+          q[k] = S.row.q[row];
+          len[k] = row_len(v, q[k], m[k]);
         }
         bin[k] = row < rows ? kLenBins - 1 - (len[k] < kLenBins ? len[k] : kLenBins - 1) : -1;
         const unsigned same = __match_any_sync(0xffffffffu, bin[k]);
@@ -446,7 +433,7 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS) k_solve(StepView v, int cls,
         const int row = S.bin[bin[k] * (NW * RPT) + sl] + rank[k];
         S.row.u[row] = u[k];
         S.row.m[row] = m[k];
-        S.row.pm0[row] = pm0[k];
+        S.row.q[row] = q[k];
         S.row.len[row] = len[k];
         v.rowof[u[k]] = row;
         v.mrow[m[k]] = row;
@@ -487,8 +474,8 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS) k_solve(StepView v, int cls,
       for (int i = 0; i < w + NW * k; ++i) sb += S.ssize[i];
       int ss = sb < ENT ? ((ENT - sb) >> 5) & ~3 : 0;
       ss = ss < sl[k].steps ? ss : sl[k].steps;
-      sl[k] = fill_slice(v, tag, lane, sl[k].len, sl[k].steps, row, u[k], on[k] ? S.row.m[row] : 0,
-                         on[k] ? S.row.pm0[row] : 0, es, sb, ss);
+      sl[k] = fill_slice(v, lane, sl[k].len, sl[k].steps, row, on[k] ? S.row.q[row] : 0, on[k] ? S.row.m[row] : 0, es,
+                         sb, ss);
     }
     group_sync<NW>();
 #pragma unroll
@@ -703,7 +690,6 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   constexpr int NW = kMultiThreads / 32;
   const unsigned lt = (1u << lane) - 1u;
-  const int tag = v.prm->tag;
   const float lam = v.lam;
   const int32_t* list = v.cls_list + (int64_t)kClsMulti * v.cls_cap;
   // rows per CTA: the total over the grid, in whole rounds of one row per thread
@@ -758,7 +744,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
           const int32_t u = v.loc2u[q];
           v.rs_u[slot0 + row] = u;
           v.rs_m[slot0 + row] = m;
-          v.rs_pm[slot0 + row] = pm0;
+          v.rs_q[slot0 + row] = q;
           v.rowof[u] = row;
           v.mrow[m] = row;
         }
@@ -786,12 +772,12 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
       const bool on = row < rows;
       const int32_t u = on ? v.rs_u[t] : 0;
       const int32_t m = on ? v.rs_m[t] : 0;
-      const int len = on ? row_len(v, tag, u, m) : 0;
+      const int32_t q = on ? v.rs_q[t] : 0;
+      const int len = on ? row_len(v, q, m) : 0;
       const int steps = slice_steps(len);
       int ss = rows <= 65536 ? kMultiSteps - used : 0;
       ss = ss < steps ? ss : steps;
-      const Slice e = fill_slice(v, tag, lane, len, steps, row, u, m, on ? v.rs_pm[t] : 0, es,
-                                 (w * kMultiSteps + used) * 32, ss);
+      const Slice e = fill_slice(v, lane, len, steps, row, q, m, es, (w * kMultiSteps + used) * 32, ss);
       used += ss;
       v.rs_len[t] = len;
       if (lane == 0) v.rs_slice[t >> 5] = make_int4(e.sb, e.ss, e.gb, e.steps);

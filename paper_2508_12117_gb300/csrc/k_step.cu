@@ -19,11 +19,10 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// Sum over the selected occurrences of pair p of vals[q] (block order).
-__device__ __forceinline__ float merge_occ(const StepView& v, int32_t p, int tag, const float* vals) {
+// Sum over the selected occurrences of a pair of vals[q], from its owner on (block order).
+__device__ __forceinline__ float merge_occ(const StepView& v, int32_t q, const float* vals) {
   float a = 0.f;
-  for (int32_t t = v.inc_off[p], t1 = v.inc_off[p + 1]; t < t1; ++t)
-    if (v.blk_stamp[v.inc_b[t]] == tag) a += vals[v.inc_q[t]];
+  for (; q >= 0; q = v.next_q[q]) a += vals[q];
   return a;
 }
 
@@ -66,17 +65,32 @@ __global__ void k_owner(StepView v) {
   int cnt = 0;
   for (int32_t q = q0 + threadIdx.x; q < q1; q += blockDim.x) {
     const int32_t p = v.node_pair[q];
-    int32_t qo = -1, bo = -1;
+    int32_t qo = -1, bo = -1, next = -1;
     int c = 0;
-    for (int32_t t = v.inc_off[p], t1 = v.inc_off[p + 1]; t < t1; ++t)
-      if (v.blk_stamp[v.inc_b[t]] == tag) {
-        if (qo < 0) {
-          qo = v.inc_q[t];
-          bo = v.inc_b[t];
-        }
-        ++c;
+    // four incidences at a time: their loads go out together
+    for (int32_t t = v.inc_off[p], t1 = v.inc_off[p + 1]; t < t1; t += 4) {
+      int32_t bb[4], qq[4];
+      bool sel[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        bb[i] = t + i < t1 ? v.inc_b[t + i] : -1;
+        qq[i] = t + i < t1 ? v.inc_q[t + i] : -1;
       }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) sel[i] = bb[i] >= 0 && v.blk_stamp[bb[i]] == tag;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (sel[i]) {
+          if (qo < 0) {
+            qo = qq[i];
+            bo = bb[i];
+          }
+          if (next < 0 && qq[i] > q) next = qq[i];      // occurrences ascend with the blocks
+          ++c;
+        }
+    }
     v.owner_q[q] = qo;
+    v.next_q[q] = next;
     if (v.owner_b) v.owner_b[q] = bo;
     v.multi[q] = (uint8_t)(c > 1);
     cnt += (qo == q);
@@ -195,28 +209,20 @@ __global__ void k_resid(StepView v) {
   }
 }
 
-// double-float sum over the selected occurrences of pair p (block order)
-__device__ __forceinline__ df32 merge_occ_df(const StepView& v, int32_t p, int tag) {
-  df32 a = {0.f, 0.f};
-  for (int32_t t = v.inc_off[p], t1 = v.inc_off[p + 1]; t < t1; ++t)
-    if (v.blk_stamp[v.inc_b[t]] == tag) {
-      const int32_t qq = v.inc_q[t];
-      a = df_add(a, df32{v.part_a[qq], v.part_c[qq]});
-    }
-  return a;
-}
-
+// u = B^T r and the diagonal of the pairs with several selected occurrences
 __global__ void k_merge_rhs(StepView v) {
-  const int tag = v.prm->tag;
   const int32_t P_u = v.counters[kCntPairs];
   for (int32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < P_u; u += gridDim.x * blockDim.x) {
-    const int32_t q = v.uniq_q[u];
-    if (!v.multi[q]) continue;
-    const int32_t p = v.node_pair[q];
-    const df32 a = merge_occ_df(v, p, tag);
+    if (!v.umulti[u]) continue;
+    df32 a = {0.f, 0.f};
+    float d = 0.f;
+    for (int32_t q = v.uniq_q[u]; q >= 0; q = v.next_q[q]) {
+      a = df_add(a, df32{v.part_a[q], v.part_c[q]});
+      d += v.part_b[q];
+    }
     v.rhs[u] = a.hi;
     v.rhs_lo[u] = a.lo;
-    v.diag[u] = v.lam + merge_occ(v, p, tag, v.part_b);
+    v.diag[u] = v.lam + d;
   }
 }
 
@@ -309,7 +315,7 @@ __global__ void k_merge_s(StepView v) {
     const int32_t m = v.pair_ev[p];
     const int sb = v.ev_sub[m];
     const float scale = (float)((double)v.sub_nobs[sb] / (double)v.sub_nsel[sb]);
-    float sp = v.multi[q] ? merge_occ(v, p, tag, v.part_a) : v.s_u[u];
+    float sp = v.multi[q] ? merge_occ(v, q, v.part_a) : v.s_u[u];
     sp *= scale;
     const float4 J = v.J[u];
     v.gp[p] = make_float4(sp * J.x, sp * J.y, sp * J.z, sp);

@@ -127,6 +127,7 @@ struct StepView {
   int32_t* sel;
   int32_t* blk_stamp;
   int32_t* owner_q;
+  int32_t* next_q;   // the pair's next selected occurrence, -1 after the last
   uint8_t* multi;
   int32_t* loc2u;
   int32_t* blk_owner_cnt;
@@ -168,6 +169,7 @@ struct StepView {
   const int64_t* piece_inv_off;   // G + 1 (null when the inverses were not built)
   const float* piece_inv;         // (lambda I + B^T B)^-1 of every piece, n x n each
   // components of the step
+  const int32_t* node_mem;        // Q: member (piece_nodes order) of a local node
   int32_t* owner_b;               // Q: block of the owner occurrence
   int32_t* plab;                  // G: piece labels
   int32_t* prow;                  // G: owner occurrences of the piece
@@ -188,7 +190,7 @@ struct StepView {
   int32_t* mrow;                  // Q: the same per member occurrence
   float2* ent;                    // 4N: matrix entries (sqrt w, column) by slice, padding included
   // row slots of the multi-CTA class
-  int32_t *rs_u, *rs_m, *rs_pm, *rs_len;
+  int32_t *rs_u, *rs_m, *rs_q, *rs_len;
   int4* rs_slice;                 // per slice: where its entries are
   float *rs_y, *rs_r, *rs_p, *rs_ap, *rs_dz, *rs_di, *rs_zh, *rs_zl;
   float4* samples;
