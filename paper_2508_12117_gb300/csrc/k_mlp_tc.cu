@@ -459,13 +459,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         {
           // product -1: the split first layer (BF16 in both forms), K = 32 of
           // K-block 0, into [H, 2H)
-          if (!mbar_wait(&a_ready[0], a_phase & 1u, abort_flag, gerr)) { ok = false; break; }
-          a_phase ^= 1u;
           const int s = (int)(n % kStages);
           if (!mbar_wait(&full[s], (uint32_t)((n / kStages) & 1), abort_flag, gerr)) { ok = false; break; }
-          tc_after();
           constexpr uint32_t idesc1 = idesc_bf16(H);
           const uint64_t bd = bdesc + (uint64_t)(s * (C::kChunk / 16));
+          if (!mbar_wait(&a_ready[0], a_phase & 1u, abort_flag, gerr)) { ok = false; break; }
+          a_phase ^= 1u;
+          tc_after();
           // A: [x_hi, x_lo, x_hi, 0 ...] in columns [16, 32) of [0, H)
           umma_ta<false>(tmem + (uint32_t)H, tmem + 16u, bd, idesc1, 0u);
           umma_ta<false>(tmem + (uint32_t)H, tmem + 24u, bd + 2, idesc1, 1u);
@@ -483,13 +483,15 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           for (int kb = 0; kb < C::KB; ++kb, ++n) {
             // K-block kb of the operand written (and the accumulator free: its last
             // reader, the epilogue two products back, finished before)
-            if (!mbar_wait(&a_ready[kb], (a_phase >> kb) & 1u, abort_flag, gerr)) { ok = false; break; }
-            a_phase ^= 1u << kb;
+            // -- after its weights, which are there first, so that nothing but the
+            // fence stands between the operand's arrival and the MMAs
             const int s = (int)(n % kStages);
             if (!mbar_wait(&full[s], (uint32_t)((n / kStages) & 1), abort_flag, gerr)) { ok = false; break; }
-            tc_after();
             const uint32_t ak = a + (uint32_t)(kb * C::kKbCols);
             const uint64_t bd = bdesc + (uint64_t)(s * (C::kChunk / 16));
+            if (!mbar_wait(&a_ready[kb], (a_phase >> kb) & 1u, abort_flag, gerr)) { ok = false; break; }
+            a_phase ^= 1u << kb;
+            tc_after();
 #pragma unroll
             for (int k = 0; k < 4; ++k)
               umma_ta<F8>(d, ak + (uint32_t)(k * C::kKstep), bd + 2 * k, idesc, (kb | k) ? 1u : 0u);
