@@ -39,17 +39,26 @@
 // a reverse layer's first stash loads are issued before its product completes).
 // At the end of a tile the first 16 columns of [0, H) carry the column groups'
 // partial sums of tau and dtau/dx to the row's first group.
-// Four weight stages hold a whole layer at H = 256 (BF16), so the next layer's
-// weights are resident when its operand is ready.
+// The weight stages hold a whole layer at H = 256, so the next layer's weights are
+// resident when its operand is ready (two stages and silu'(z2) in shared memory in
+// the BF16 form: 1365 -> 1453 us at 1.57 M pairs).  What is left at H = 256 is the
+// chain from one product to the next, not any one unit: finer barriers (one per
+// K-step, 1490 us) or an arrival half a chunk later (1489) both cost more.
+// 1.57 M pairs BF16: 1352 us, 919 TFLOP/s.
 // Shared memory keeps W1 and the biases pre-halved (exact): the epilogue works
 // with u = z/2, silu(z) = u + u tanh(u), silu'(z) = s + silu(z) (1 - s),
 // s = (1 + tanh(u)) / 2.
 // FP8 form (kind::f8f6f4, E4M3 operands, FP32 accumulation): the weight images
 // carry one scale per output column (max |W| / 448); each activation row is
-// quantised with its own scale, from a first pass over the accumulator that
-// bounds the row's largest magnitude (the four threads holding a row exchange
-// their bounds through a 128-arrival mbarrier); delta4 = w5 * silu'(z4)
-// uses the fixed bound 1.1 max |w5|.  The accumulator of the next layer is
+// quantised with its own scale, from a bound of the row's largest magnitude that
+// the epilogue takes while it forms the operand.  The operand waits in FP32 in the
+// accumulator's columns until the four threads holding a row have exchanged
+// their bounds through an mbarrier, then is read back, scaled and packed.  (A
+// first pass over the accumulator for the bound alone repeated the
+// dequantisation, one value at a time: 400,003 pairs at H = 256 took 563 us, now
+// 513 with silu'(z2) in the shared memory of two weight stages, which a layer of
+// two K-blocks does not need; BF16 at the same size takes about 350.)  delta4 =
+// w5 * silu'(z4) uses the fixed bound 1.1 max |w5|.  The accumulator of the next layer is
 // rescaled by (row scale) x (column scale) before bias and activation.
 // Every wait is bounded (2 s on the global timer): on timeout the kernel sets
 // SPIDER_E_TIMEOUT, drains its own copies and MMAs, frees TMEM and returns.
@@ -97,18 +106,24 @@ struct Cfg {
   static_assert(KB <= kMaxKb && kChunks == KB * kCpk && kCpk >= 1, "tile shape");
   static constexpr int kTmemCols = 2 * H;
   static constexpr int kChunksPerTile = 1 + 6 * KB;  // the first layer's image (one K-block), then 6 layers
+  // Weight stages: a whole layer (H = 256: four K-blocks in BF16, two in FP8,
+  // where the room of two more holds silu'(z2))
+  static constexpr int kSt = F8 && H >= 256 ? 2 : kStages;
   // shared-memory carve-up (offsets from a 1024-aligned base)
   static constexpr int oB = 0;
-  static constexpr int oPar = oB + kStages * kChunk;      // W1 (6H), b1, b2, b3, b4, w5 (5H) floats
-  static constexpr int oSc = oPar + 11 * H * 4;           // FP8: column scales of the 6 images (6H floats)
-  static constexpr int oXch = oSc + (F8 ? 6 * H * 4 : 0); // FP8: row-bound exchange [2][kGroups][kRows] floats
-  static constexpr int oGeo = oXch + (F8 ? 2 * kGroups * kRows * 4 : 0);   // pair geometry [2][15][kRows] floats
+  static constexpr int oPar = oB + kSt * kChunk;          // W1[:, :3] (3H), b1, b2, b3, b4, w5 (5H) floats
+  static constexpr int oSc = oPar + 8 * H * 4;           // FP8: column scales of the 6 images (6H floats)
+  static constexpr int oXch = oSc + (F8 ? 6 * H * 4 : 0); // FP8: row-bound exchange [kGroups][kRows] floats
+  static constexpr int oGeo = oXch + (F8 ? kGroups * kRows * 4 : 0);   // pair geometry [2][15][kRows] floats
   // silu'(z3) of the current tile (kD bytes) in shared memory when it fits
   // (read by the first reverse layer, two products after it is written);
   // otherwise it goes to the third global slot like silu'(z1), silu'(z2)
   static constexpr int oD3 = oGeo + 2 * 15 * kRows * 4;
   static constexpr bool kD3Shared = oD3 + kD + kBars * 8 + 16 + 1024 <= 232448;
-  static constexpr int oBar = oD3 + (kD3Shared ? kD : 0);         // mbarriers
+  // likewise silu'(z2) in the FP8 form
+  static constexpr int oD2 = oD3 + (kD3Shared ? kD : 0);
+  static constexpr bool kD2Shared = F8 && kD3Shared && oD2 + kD + kBars * 8 + 16 + 1024 <= 232448;
+  static constexpr int oBar = oD2 + (kD2Shared ? kD : 0);         // mbarriers
   static constexpr int oMisc = oBar + kBars * 8;          // tmem base, abort flag
   static constexpr int kSmem = oMisc + 16 + 1024;         // + alignment slack
   static_assert(kSmem <= 232448, "shared memory per CTA");
@@ -230,6 +245,15 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8])
                "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
                : "memory");
 }
+__device__ __forceinline__ void tmem_st16f(uint32_t taddr, const float (&v)[16]) {
+  const uint32_t* r = reinterpret_cast<const uint32_t*>(v);
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+      "%15, %16};" ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+      : "memory");
+}
 __device__ __forceinline__ void tmem_ld16f(uint32_t taddr, float (&v)[16]) {
   uint32_t* r = reinterpret_cast<uint32_t*>(v);
   asm volatile(
@@ -299,18 +323,20 @@ __device__ __forceinline__ uint32_t pack_e4m3x4(float a, float b, float c, float
 }
 
 // FP8: largest magnitude bound of a row over its column groups (bounded wait);
-// every thread of the row takes the maximum in the same order
+// every thread of the row takes the maximum in the same order.  One buffer: the
+// next exchange comes after the next product, which waits for every warp's
+// operand, written after that warp read this one.
 __device__ __forceinline__ bool group_max(float& m, float* xch, uint64_t* xbar, uint32_t& xph, int cg, int r,
                                           volatile int* abort_flag, int32_t* gerr) {
-  const int slot = (int)(xph & 1);
-  xch[(slot * kGroups + cg) * kRows + r] = m;
-  mbar_arrive(xbar);
-  const bool got = mbar_wait(xbar, xph & 1, abort_flag, gerr);
+  xch[cg * kRows + r] = m;
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(xbar);
+  const bool got = mbar_wait(xbar, xph, abort_flag, gerr);
   xph ^= 1;
   if (got) {
-    float a = xch[(slot * kGroups) * kRows + r];
+    float a = xch[r];
 #pragma unroll
-    for (int q = 1; q < kGroups; ++q) a = fmaxf(a, xch[(slot * kGroups + q) * kRows + r]);
+    for (int q = 1; q < kGroups; ++q) a = fmaxf(a, xch[q * kRows + r]);
     m = a;
   }
   return got;
@@ -335,7 +361,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   uint8_t* sD = stash + (size_t)blockIdx.x * C::kStash;
   uint8_t* sD3 = C::kD3Shared ? sm + C::oD3 : sD + 2 * (size_t)C::kD;   // the slot of silu'(z3)
   float* pW1 = reinterpret_cast<float*>(sm + C::oPar);
-  float* pb1 = pW1 + 6 * H;
+  float* pb1 = pW1 + 3 * H;
   float* pb = pb1 + H;       // b2, b3, b4
   float* pw5 = pb + 3 * H;
   float* wsc = reinterpret_cast<float*>(sm + C::oSc);     // FP8 column scales [6][H]
@@ -364,7 +390,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     for (int q = 0; q < kMaxKb; ++q) mbar_init(&a_ready[q], kEpiWarps);
     mbar_init(drain, 1);
     mbar_init(red_ready, kEpiThreads);
-    for (int q = 0; q < 4; ++q) mbar_init(&xbar[q], 32 * kGroups);
+    for (int q = 0; q < 4; ++q) mbar_init(&xbar[q], kGroups);
     for (int q = 0; q < 2; ++q) {
       mbar_init(&geo_full[q], 32);
       mbar_init(&geo_empty[q], kEpiThreads);
@@ -372,9 +398,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // W1 / 2 transposed in shared memory (6 x H: input c, column) so that column
-  // pairs are adjacent; b1 / 2 .. b4 / 2 (halving is exact)
-  for (int i = threadIdx.x; i < 6 * H; i += blockDim.x) pW1[(i % 6) * H + i / 6] = 0.5f * net.W1[i];
+  // W1[:, :3] / 2 transposed in shared memory (3 x H: input c, column) so that
+  // column pairs are adjacent; b1 / 2 .. b4 / 2 (halving is exact)
+  for (int i = threadIdx.x; i < 3 * H; i += blockDim.x) pW1[(i % 3) * H + i / 3] = 0.5f * net.W1[(i / 3) * 6 + i % 3];
   for (int i = threadIdx.x; i < H; i += blockDim.x) {
     pb1[i] = 0.5f * net.b1[i];
     pb[i] = 0.5f * net.bh[0][i];
@@ -404,8 +430,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       const int64_t total = my_tiles * C::kChunksPerTile;
       int64_t n = 0;
       for (; n < total; ++n) {
-        const int s = (int)(n % kStages);
-        const int64_t use = n / kStages;
+        const int s = (int)(n % C::kSt);
+        const int64_t use = n / C::kSt;
         if (use > 0 && !mbar_wait(&empty[s], (uint32_t)((use - 1) & 1), abort_flag, gerr)) break;
         // the images are stored in consumption order, K-block after K-block
         const int c = (int)(n % C::kChunksPerTile);
@@ -414,10 +440,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         bulk_load(sB + s * C::kChunk, g, C::kChunk, &full[s]);
       }
       // copies still in flight must land before the CTA's shared memory goes away
-      for (int64_t m = (n > kStages ? n - kStages : 0); m < n; ++m) {
-        const int s = (int)(m % kStages);
+      for (int64_t m = (n > C::kSt ? n - C::kSt : 0); m < n; ++m) {
+        const int s = (int)(m % C::kSt);
         const uint64_t t0 = gtime();
-        while (!mbar_test(&full[s], (uint32_t)((m / kStages) & 1)))
+        while (!mbar_test(&full[s], (uint32_t)((m / C::kSt) & 1)))
           if (gtime() - t0 > kWaitNs) break;
       }
     }
@@ -459,8 +485,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         {
           // product -1: the split first layer (BF16 in both forms), K = 32 of
           // K-block 0, into [H, 2H)
-          const int s = (int)(n % kStages);
-          if (!mbar_wait(&full[s], (uint32_t)((n / kStages) & 1), abort_flag, gerr)) { ok = false; break; }
+          const int s = (int)(n % C::kSt);
+          if (!mbar_wait(&full[s], (uint32_t)((n / C::kSt) & 1), abort_flag, gerr)) { ok = false; break; }
           constexpr uint32_t idesc1 = idesc_bf16(H);
           const uint64_t bd = bdesc + (uint64_t)(s * (C::kChunk / 16));
           if (!mbar_wait(&a_ready[0], a_phase & 1u, abort_flag, gerr)) { ok = false; break; }
@@ -485,8 +511,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             // reader, the epilogue two products back, finished before)
             // -- after its weights, which are there first, so that nothing but the
             // fence stands between the operand's arrival and the MMAs
-            const int s = (int)(n % kStages);
-            if (!mbar_wait(&full[s], (uint32_t)((n / kStages) & 1), abort_flag, gerr)) { ok = false; break; }
+            const int s = (int)(n % C::kSt);
+            if (!mbar_wait(&full[s], (uint32_t)((n / C::kSt) & 1), abort_flag, gerr)) { ok = false; break; }
             const uint32_t ak = a + (uint32_t)(kb * C::kKbCols);
             const uint64_t bd = bdesc + (uint64_t)(s * (C::kChunk / 16));
             if (!mbar_wait(&a_ready[kb], (a_phase >> kb) & 1u, abort_flag, gerr)) { ok = false; break; }
@@ -548,9 +574,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     };
     // silu'(z_q), q = 1, 2, 3, of columns col .. col + 15 into slot q
     auto put_d = [&](int q, int col, const uint32_t (&dp)[kCc / 2]) {
-      uint8_t* b = q == 3 ? sD3 : sD + (size_t)(q - 1) * C::kD;
-      *reinterpret_cast<uint4*>(b + d_off(r, col)) = make_uint4(dp[0], dp[1], dp[2], dp[3]);
-      *reinterpret_cast<uint4*>(b + d_off(r, col + 8)) = make_uint4(dp[4], dp[5], dp[6], dp[7]);
+      const uint4 lo = make_uint4(dp[0], dp[1], dp[2], dp[3]), hi = make_uint4(dp[4], dp[5], dp[6], dp[7]);
+      auto put = [&](uint8_t* b) {
+        *reinterpret_cast<uint4*>(b + d_off(r, col)) = lo;
+        *reinterpret_cast<uint4*>(b + d_off(r, col + 8)) = hi;
+      };
+      if constexpr (C::kD2Shared) {
+        if (q >= 2) put(sm + (q == 2 ? C::oD2 : C::oD3)); else put(sD);
+      } else {
+        put(q == 3 ? sD3 : sD + (size_t)(q - 1) * C::kD);
+      }
     };
     uint32_t acc_phase = 0, red_phase = 0, xph = 0;
     for (int64_t t = 0; t < my_tiles; ++t) {
@@ -609,13 +642,21 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         // MMA); chunk j + kPre is requested while chunk j is processed
         constexpr int kPre = C::kChunks < 2 ? C::kChunks : 2;
         const uint8_t* dsl = layer == 3 ? sD3 : sD + (size_t)(layer >= 3 ? 5 - layer : 0) * C::kD;
+        auto get_d = [&](int col, uint4& lo, uint4& hi) {
+          auto get = [&](const uint8_t* b) {
+            lo = *reinterpret_cast<const uint4*>(b + d_off(r, col));
+            hi = *reinterpret_cast<const uint4*>(b + d_off(r, col + 8));
+          };
+          if constexpr (C::kD2Shared) {
+            if (layer < 5) get(sm + (layer == 4 ? C::oD2 : C::oD3)); else get(sD);
+          } else {
+            get(dsl);
+          }
+        };
         uint4 dsv[2 * kPre];
         if (layer >= 3) {
 #pragma unroll
-          for (int j = 0; j < kPre; ++j) {
-            dsv[2 * j] = *reinterpret_cast<const uint4*>(dsl + d_off(r, ccol(j)));
-            dsv[2 * j + 1] = *reinterpret_cast<const uint4*>(dsl + d_off(r, ccol(j) + 8));
-          }
+          for (int j = 0; j < kPre; ++j) get_d(ccol(j), dsv[2 * j], dsv[2 * j + 1]);
         }
         const bool got = mbar_wait(acc_ready, acc_phase, abort_flag, gerr);
         if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
@@ -623,38 +664,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         tc_after();
         const uint32_t acc = lane_addr + (uint32_t)((layer & 1) * H);   // this product's accumulator
         // FP8: dequantisation of the accumulator, (row scale) x (column scale); the
-        // first layer's BF16 product needs none
+        // first layer's BF16 product needs none.  The operand's scale is fixed for
+        // delta4; otherwise it follows from a bound of the whole row (silu(z)
+        // forward, delta backward), which this pass takes while it forms the operand
+        // and leaves it in FP32 in the accumulator's columns; a second pass scales
+        // and packs it once the row's threads have met.
         const float* sw = wsc + (layer > 0 ? layer : 0) * H;
-        const float sa_l = layer < 0 ? 0.f : sa;
-        auto dq = [&](int c) { return layer < 0 ? 1.f : sa_l * sw[c]; };
-        float inv = 1.f, sa_next = sa;
-        if constexpr (F8) {
-          if (layer == -1 || layer == 0 || layer == 1 || layer == 3 || layer == 4) {
-            // bound of the row for the next A operand (silu(z) forward, delta backward)
-            const float* bias = pb + layer * H;
-            float m = layer <= 1 ? 0.2785f : 1e-30f;
-            for (int j = 0; j < C::kChunks; ++j) {
-              const int col = ccol(j);
-              float v[kCc];
-              tmem_ld16f(acc + col, v);
-              tmem_wait_ld();
-              if (layer <= 1) {
-#pragma unroll
-                for (int i = 0; i < kCc; ++i) m = fmaxf(m, 2.f * fmaf(v[i] * dq(col + i), 0.5f, bias[col + i]));
-              } else {
-#pragma unroll
-                for (int i = 0; i < kCc; ++i) m = fmaxf(m, 1.1f * fabsf(v[i] * dq(col + i)));
-              }
-            }
-            const bool got2 = group_max(m, xch, &xbar[g], xph, cg, r, abort_flag, gerr);
-            if (!__all_sync(0xffffffffu, got2)) { ok = false; break; }
-            inv = 448.f / m;
-            sa_next = m / 448.f;
-          } else if (layer == 2) {
-            inv = 1.f / s4;
-            sa_next = s4;
-          }
-        }
+        const uint64_t sa2 = f2pack(sa, sa);
+        const bool two = layer < 5 && layer != 2;
+        float m = layer <= 1 ? 0.2785f : 1e-30f;
+        const float inv = F8 && layer == 2 ? 1.f / s4 : 1.f;
         // chunk j + 1 is read from TMEM while chunk j is processed (two register
         // buffers; tcgen05.wait::ld at the end of chunk j waits for that one read)
         float vb[2][kCc];
@@ -666,8 +685,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           if (j + 1 < C::kChunks) tmem_ld16f(acc + ccol(j + 1), vb[(j + 1) & 1]);
           float* v = vb[j & 1];
           if constexpr (F8) {
+            if (layer >= 0) {
 #pragma unroll
-            for (int i = 0; i < kCc; ++i) v[i] *= dq(col + i);
+              for (int i = 0; i < kCc; i += 4) {
+                const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(sw + col + i);
+                f2unpack(f2mul(f2pack(v[i], v[i + 1]), f2mul(sa2, w.x)), v[i], v[i + 1]);
+                f2unpack(f2mul(f2pack(v[i + 2], v[i + 3]), f2mul(sa2, w.y)), v[i + 2], v[i + 3]);
+              }
+            }
           }
           float o[kCc];                                // next A operand values (unscaled)
           if (layer < 3) {
@@ -678,8 +703,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             for (int i = 0; i < kCc; i += 4) {
               const float4 b4 = *reinterpret_cast<const float4*>(bias + col + i);
               uint64_t hh[2], dd2[2];
-              silu_half(f2fma(f2pack(v[i], v[i + 1]), kHalf2, f2pack(b4.x, b4.y)), hh[0], dd2[0]);
-              silu_half(f2fma(f2pack(v[i + 2], v[i + 3]), kHalf2, f2pack(b4.z, b4.w)), hh[1], dd2[1]);
+              const uint64_t ua = f2fma(f2pack(v[i], v[i + 1]), kHalf2, f2pack(b4.x, b4.y));
+              const uint64_t ub = f2fma(f2pack(v[i + 2], v[i + 3]), kHalf2, f2pack(b4.z, b4.w));
+              if constexpr (F8) {
+                float u0, u1, u2, u3;
+                f2unpack(ua, u0, u1);
+                f2unpack(ub, u2, u3);
+                m = fmaxf(fmaxf(m, 2.f * fmaxf(u0, u1)), 2.f * fmaxf(u2, u3));
+              }
+              silu_half(ua, hh[0], dd2[0]);
+              silu_half(ub, hh[1], dd2[1]);
 #pragma unroll
               for (int q = 0; q < 2; ++q) {
                 const int ii = i + 2 * q;
@@ -703,13 +736,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             if (layer < 2) put_d(layer + 2, col, dp);  // silu'(z1), silu'(z2), silu'(z3)
           } else {
             // reverse sweep: delta_{l-1} = acc * silu'(z_{l-1})
+            if constexpr (F8) {
+#pragma unroll
+              for (int i = 0; i < kCc; i += 2) m = fmaxf(m, 1.1f * fmaxf(fabsf(v[i]), fabsf(v[i + 1])));
+            }
             const int sl = j % kPre;
             const uint32_t dd[8] = {dsv[2 * sl].x, dsv[2 * sl].y, dsv[2 * sl].z, dsv[2 * sl].w,
                                     dsv[2 * sl + 1].x, dsv[2 * sl + 1].y, dsv[2 * sl + 1].z, dsv[2 * sl + 1].w};
-            if (j + kPre < C::kChunks) {
-              dsv[2 * sl] = *reinterpret_cast<const uint4*>(dsl + d_off(r, ccol(j + kPre)));
-              dsv[2 * sl + 1] = *reinterpret_cast<const uint4*>(dsl + d_off(r, ccol(j + kPre) + 8));
-            }
+            if (j + kPre < C::kChunks) get_d(ccol(j + kPre), dsv[2 * sl], dsv[2 * sl + 1]);
 #pragma unroll
             for (int i = 0; i < kCc; i += 2)
               f2unpack(f2mul(f2pack(v[i], v[i + 1]), f2pack(bf16_lo(dd[i / 2]), bf16_hi(dd[i / 2]))), o[i],
@@ -732,14 +766,34 @@ __global__ void __launch_bounds__(kTcThreads, 1)
               }
             }
           }
-          if (layer < 5) {
+          if (F8 && two) {
+            tmem_st16f(acc + col, o);
+          } else if (layer < 5) {
             put_a(acc, col, o, inv);
             if ((j + 1) % C::kCpk == 0) a_done(j / C::kCpk);
           }
           if (j + 1 < C::kChunks) tmem_wait_ld();
         }
-        if (!ok) break;
-        sa = sa_next;
+        if constexpr (F8) {
+          if (two) {
+            const bool got2 = group_max(m, xch, &xbar[g], xph, cg, r, abort_flag, gerr);
+            if (!__all_sync(0xffffffffu, got2)) { ok = false; break; }
+            const float inv2 = 448.f / m;
+            sa = m / 448.f;
+            tmem_wait_st();
+            tmem_ld16f(acc + ccol(0), vb[0]);
+            tmem_wait_ld();
+#pragma unroll
+            for (int j = 0; j < C::kChunks; ++j) {
+              if (j + 1 < C::kChunks) tmem_ld16f(acc + ccol(j + 1), vb[(j + 1) & 1]);
+              put_a(acc, ccol(j), vb[j & 1], inv2);
+              if (j + 1 < C::kChunks) tmem_wait_ld();
+              if ((j + 1) % C::kCpk == 0) a_done(j / C::kCpk);
+            }
+          } else if (layer == 2) {
+            sa = s4;
+          }
+        }
       }
       if (!ok) break;
       // combine the column groups of each row (fixed order) and write T, dT/dx:
