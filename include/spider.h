@@ -357,6 +357,12 @@ void spider_net_free(spider_netdev *nd);
 int spider_tt_pairs(const spider_netdev *nd, int64_t P, const float *src, const float *rcv,
                     float *T_hi, float *T_lo, float *J, void *stream);
 
+/* The same for positions in rows of three (device P x 3 FP32, no padding), with
+ * T = T_hi + T_lo rounded to FP32.  T and J overlap neither each other nor the
+ * positions. */
+int spider_tt_pairs_rows(const spider_netdev *nd, int64_t P, const float *src, const float *rcv,
+                         float *T, float *J, void *stream);
+
 /* Allocation-free variant of spider_tt_pairs for the MLP model in FP32.  The
  * paper has no counterpart: it exists for callers that may not allocate device
  * memory -- code running inside a runtime that owns all device memory up

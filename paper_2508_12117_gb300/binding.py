@@ -104,6 +104,7 @@ def load_library(path: str = LIB_PATH):
         "spider_net_free": (None, [vp]),
         "spider_tt_pairs": (C.c_int, [vp, i64, vp, vp, vp, vp, vp, vp]),
         "spider_philox_words": (C.c_int, [u64, u32, u32, u32, u32, i64, C.POINTER(u32)]),
+        "spider_tt_pairs_rows": (C.c_int, [vp, i64, vp, vp, vp, vp, vp]),
         "spider_tt_pairs_noalloc": (C.c_int, [C.POINTER(spider_net), i64, vp, vp, vp, vp, vp, vp]),
     }
     for name, (res, args) in sig.items():
@@ -453,6 +454,14 @@ class NetDevice:
         _check(load_library().spider_tt_pairs(self.h, P, C.c_void_p(src_ptr), C.c_void_p(rcv_ptr),
                                               C.c_void_p(thi_ptr), C.c_void_p(tlo_ptr or None),
                                               C.c_void_p(j_ptr or None), C.c_void_p(stream or None)),
+               None)
+
+
+    def spider_tt_pairs_rows(self, P: int, src_ptr: int, rcv_ptr: int, t_ptr: int, j_ptr: int, stream: int = 0):
+        """The same for positions in rows of three, with T rounded to FP32."""
+        _check(load_library().spider_tt_pairs_rows(self.h, P, C.c_void_p(src_ptr), C.c_void_p(rcv_ptr),
+                                                   C.c_void_p(t_ptr), C.c_void_p(j_ptr or None),
+                                                   C.c_void_p(stream or None)),
                None)
 
 

@@ -1349,6 +1349,23 @@ int spider_tt_pairs(const spider_netdev* nd, int64_t P, const float* src, const 
   return SPIDER_OK;
 }
 
+int spider_tt_pairs_rows(const spider_netdev* nd, int64_t P, const float* src, const float* rcv, float* T, float* J,
+                         void* stream) {
+  if (!nd || P < 0 || P > (int64_t)INT32_MAX || (P > 0 && (!src || !rcv || !T))) return SPIDER_E_INVAL;
+  if (P == 0) return SPIDER_OK;
+  PairSource ps{};
+  ps.src3 = src;
+  ps.rcv3 = rcv;
+  ps.n_host = P;
+  const TTOut out{nullptr, reinterpret_cast<float4*>(J), T, nullptr, true};
+  const cudaError_t e = launch_tt(nd->net, ps, out, nd->num_sms, nd->scratch, (cudaStream_t)stream, 2);
+  if (e != cudaSuccess) {
+    g_static_err = cudaGetErrorString(e);
+    return SPIDER_E_CUDA;
+  }
+  return SPIDER_OK;
+}
+
 int spider_philox_words(uint64_t seed, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, int64_t n,
                         uint32_t* out) {
   if (n < 0 || (n > 0 && !out) || n > (int64_t(1) << 28)) return SPIDER_E_INVAL;

@@ -26,9 +26,17 @@ __device__ __forceinline__ void load_pair(const PairSource& s, int64_t u, PairGe
     g.rhi[0] = c.x; g.rhi[1] = c.y; g.rhi[2] = c.z;
     g.rlo[0] = e.x; g.rlo[1] = e.y; g.rlo[2] = e.z;
   } else {
-    const float4 a = s.src[u], c = s.rcv[u];
-    g.shi[0] = a.x; g.shi[1] = a.y; g.shi[2] = a.z;
-    g.rhi[0] = c.x; g.rhi[1] = c.y; g.rhi[2] = c.z;
+    if (s.src) {
+      const float4 a = s.src[u], c = s.rcv[u];
+      g.shi[0] = a.x; g.shi[1] = a.y; g.shi[2] = a.z;
+      g.rhi[0] = c.x; g.rhi[1] = c.y; g.rhi[2] = c.z;
+    } else {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        g.shi[i] = s.src3[3 * u + i];
+        g.rhi[i] = s.rcv3[3 * u + i];
+      }
+    }
 #pragma unroll
     for (int i = 0; i < 3; ++i) g.slo[i] = g.soff[i] = g.rlo[i] = 0.f;
   }
@@ -38,7 +46,7 @@ __device__ __forceinline__ void store_time(const TTOut& o, int64_t u, float hi, 
   if (o.T2) {
     o.T2[u] = make_float2(hi, lo);
   } else {
-    o.hi[u] = hi;
+    o.hi[u] = o.sum ? hi + lo : hi;
     if (o.lo) o.lo[u] = lo;
   }
 }

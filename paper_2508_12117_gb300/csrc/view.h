@@ -53,6 +53,8 @@ struct PairSource {
   // raw mode (uniq_pair == nullptr): absolute FP32 positions per pair
   const float4* src;
   const float4* rcv;
+  const float* src3;      // the same as rows of three (src == nullptr)
+  const float* rcv3;
   const int32_t* n_dev;   // device count (problem mode) or nullptr
   int64_t n_host;         // host count (raw mode) / upper bound
 };
@@ -62,6 +64,7 @@ struct TTOut {
   float4* J;    // (dT/dx, dT/dy, dT/dz, 0), may be null
   float* hi;
   float* lo;
+  bool sum;     // hi takes T_hi + T_lo rounded
 };
 
 // Per-step parameters, read by the kernels from device memory (the host
