@@ -493,6 +493,18 @@ int build_whitening(spider_ctx* c, const Prep& P, bool want_inverses) {
     c->err = "whitening kernels do not fit on the device";
     return SPIDER_E_UNSUPPORTED;
   }
+  {
+    // a component lies in one station of one sub-problem: the most pairs and pieces of one
+    std::vector<int32_t> pairs((size_t)P.n_sub * P.S, 0), pieces(pairs.size(), 0);
+    auto at = [&](int32_t p) { return (size_t)P.ev_sub[P.pair_ev[p]] * P.S + P.pair_st[p]; };
+    for (int64_t p = 0; p < P.P; ++p) ++pairs[at((int32_t)p)];
+    for (int64_t b = 0; b < P.NB; ++b)
+      for (int32_t g = T.blk_piece_off[b]; g < T.blk_piece_off[b + 1]; ++g)
+        ++pieces[at(P.node_pair[P.blk_node_off[b] + T.piece_nodes[T.piece_node_off[g]]])];
+    c->plan.top_class = kClsWarp;
+    for (size_t k = 0; k < pairs.size(); ++k)
+      c->plan.top_class = std::max(c->plan.top_class, (int)solve_class(pairs[k], pieces[k]));
+  }
   if ((e = cudaEventCreateWithFlags(&c->ubr.fork, cudaEventDisableTiming))) return cuda_fail(c, e, "event");
   for (int i = 0; i < kBranches; ++i) {
     if ((e = cudaStreamCreateWithFlags(&c->ubr.s[i], cudaStreamNonBlocking))) return cuda_fail(c, e, "branch stream");

@@ -16,10 +16,14 @@
 // ascending piece id and member order, so their order, and with it every sum,
 // does not depend on how lists were filled.  A row belongs to one lane; the
 // entries of the 32 rows of a slice are stored step by step (the t-th entries
-// of all rows side by side), so a warp's loads are contiguous, and the gathered neighbours of consecutive rows (the same
-// event at consecutive stations) are mostly contiguous too.  One thread per
+// of all rows side by side), so a warp's loads are contiguous.  One thread per
 // row over row-contiguous entries touched 32 cache lines per load and was
 // bound by the load unit (48 us per iteration over 110 k rows and 4 M entries).
+//
+// Measured and left out: clusters of two and four CTAs that write their y into
+// each other's shared memory.  A component of 700 rows took 3100 cycles an
+// iteration on two CTAs, 3400 on one, and clusters, which wait for whole SMs at once, started
+// after every smaller class: steps with many components lost 5-30 %.
 #include <cuda_runtime.h>
 
 #include "dfloat.cuh"
@@ -71,6 +75,7 @@ __device__ __forceinline__ int slice_steps(int len) { return ((int)__reduce_max_
 // (lane = row of `len` entries, 0 where there is none), its first ss steps to
 // shared memory and the others to a range taken from the pool.  A row's entries
 // run over its occurrences in block order, then in observation order.
+template <int kFill>
 __device__ __forceinline__ Slice fill_slice(const StepView& v, int lane, int len, int steps, int row, int32_t q,
                                             int32_t m, EntrySmem es, int sb, int ss) {
   const unsigned lt = (1u << lane) - 1u;
@@ -89,11 +94,13 @@ __device__ __forceinline__ Slice fill_slice(const StepView& v, int lane, int len
     at = __shfl_sync(0xffffffffu, at, 0);
     s.gb = padded ? at : ~at;
   }
-  for (int j = 0; j < steps; j += 4) {
-    int32_t pos[4], ei[4], pm[4];
+  // kFill entries at a time: three dependent trips to L2 each (8 instead of 4 saves a
+  // tenth of a component's time); steps is a multiple of 4
+  for (int j = 0; j < steps; j += kFill) {
+    int32_t pos[kFill], ei[kFill], pm[kFill];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (j < ss) {
+    for (int i = 0; i < kFill; ++i) {
+      if (j + i < ss) {
         pos[i] = sb + 32 * (j + i) + lane;
       } else if (padded) {
         pos[i] = at + 32 * (j - ss + i) + lane;
@@ -116,10 +123,10 @@ __device__ __forceinline__ Slice fill_slice(const StepView& v, int lane, int len
         pm[i] = pm0;
       }
     }
-    float sw[4];
-    int32_t col[4];
+    float sw[kFill];
+    int32_t col[kFill];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < kFill; ++i) {
       sw[i] = 0.f;
       col[i] = -1;
       if (j + i < len) {
@@ -128,10 +135,11 @@ __device__ __forceinline__ Slice fill_slice(const StepView& v, int lane, int len
       }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) col[i] = col[i] >= 0 ? v.mrow[col[i]] : row;
+    for (int i = 0; i < kFill; ++i) col[i] = col[i] >= 0 ? v.mrow[col[i]] : row;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (j < ss) {
+    for (int i = 0; i < kFill; ++i) {
+      if (j + i >= steps) break;
+      if (j + i < ss) {
         es.sw[pos[i]] = sw[i];
         es.col[pos[i]] = (uint16_t)col[i];
       } else if (padded || j + i < len) {
@@ -142,15 +150,51 @@ __device__ __forceinline__ Slice fill_slice(const StepView& v, int lane, int len
   return s;
 }
 
+// The first K steps of a slice in registers: weights w = sw^2, columns in pairs.
+template <int K>
+struct Held {
+  float w[K > 0 ? K : 1];
+  uint32_t c[K > 0 ? K / 2 : 1];
+};
+
+template <int K>
+__device__ __forceinline__ void hold(Held<K>& h, EntrySmem es, const Slice& sl, int lane) {
+  const float* ws = es.sw + sl.sb + lane;
+  const uint16_t* cs = es.col + sl.sb + lane;
+#pragma unroll
+  for (int j = 0; j < K; j += 2) {
+    const bool in = j < sl.ss;
+    const float a = in ? ws[32 * j] : 0.f, b = in ? ws[32 * j + 32] : 0.f;
+    h.w[j] = a * a;
+    h.w[j + 1] = b * b;
+    h.c[j / 2] = in ? (uint32_t)cs[32 * j] | ((uint32_t)cs[32 * j + 32] << 16) : 0u;
+  }
+}
+
 // sum over the row's entries of w (y_row - y_col), w = sw^2
-__device__ __forceinline__ float slice_mul(const float2* ent, EntrySmem es, const Slice& sl, int lane, float yr,
-                                           const float* y) {
+template <int K>
+__device__ __forceinline__ float slice_mul(const float2* ent, EntrySmem es, const Slice& sl, const Held<K>& h, int lane,
+                                           float yr, const float* y) {
   float s = 0.f;
+#pragma unroll
+  for (int j = 0; j < K; j += 4) {
+    if (j < sl.ss) {
+      float t[4];
+#pragma unroll
+      for (int i = 0; i < 4; i += 2) {
+        t[i] = y[h.c[(j + i) / 2] & 0xFFFFu];
+        t[i + 1] = y[h.c[(j + i) / 2] >> 16];
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s = fmaf(h.w[j + i], yr - t[i], s);
+    }
+  }
+  if (sl.steps <= K && sl.ss == sl.steps) return s;
   {
-    const float* ws = es.sw + sl.sb + lane;
-    const uint16_t* cs = es.col + sl.sb + lane;
+    const float* ws = es.sw + sl.sb + lane + 32 * K;
+    const uint16_t* cs = es.col + sl.sb + lane + 32 * K;
 #pragma unroll 2
-    for (int j = 0; j < sl.ss; j += 4, ws += 4 * 32, cs += 4 * 32) {
+    for (int j = K; j < sl.ss; j += 4, ws += 4 * 32, cs += 4 * 32) {
       float w[4];
       int c[4];
 #pragma unroll
@@ -265,10 +309,26 @@ __device__ __forceinline__ float2 group_sum2(float a, float b, float2* part, int
   } else {
     if (lane == 0) part[par * NW + w] = s;
     __syncthreads();
-    s = part[par * NW + (lane & (NW - 1))];
+    // every lane adds eight warps' sums (four at 32 warps, where the reads would
+    // take longer than the shuffles), the rest by shuffles
+    constexpr int E = NW > 16 ? 4 : 8;
+    const float4* q = reinterpret_cast<const float4*>(part + par * NW + (lane & (NW / E - 1)) * E);
+    float4 x[E / 2];
+#pragma unroll
+    for (int i = 0; i < E / 2; ++i) x[i] = q[i];
+#pragma unroll
+    for (int h = E / 4; h > 0; h >>= 1)
+#pragma unroll
+      for (int i = 0; i < h; ++i) {
+        x[i].x += x[i + h].x;
+        x[i].y += x[i + h].y;
+        x[i].z += x[i + h].z;
+        x[i].w += x[i + h].w;
+      }
+    s = make_float2(x[0].x + x[0].z, x[0].y + x[0].w);
     par ^= 1;
 #pragma unroll
-    for (int o = NW / 2; o > 0; o >>= 1) {
+    for (int o = NW / E / 2; o > 0; o >>= 1) {
       s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
       s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
     }
@@ -298,7 +358,7 @@ struct SolveSmem {
     };
     int32_t bin[kLenBins * NW * RPT];       // rows per length and slice
   };
-  float2 part[2 * NW];
+  alignas(16) float2 part[2 * NW];
   int32_t wsum[NW], ssize[NW * RPT];
   int32_t unit;
 };
@@ -339,8 +399,18 @@ __device__ void group_exscan(int32_t* a, int32_t* wsum, int tid, int w, int lane
 // ENT: matrix entries per component in shared memory (6 bytes each, longest
 // slices first).  Through L1 they were evicted by the clean pieces' solver, which
 // streams its inverses on the same SMs: 770 cycles per four steps instead of ~100.
-template <int NW, int RPT, int GROUPS, int KP, int ENT>
-__global__ void __launch_bounds__(NW * 32 * GROUPS) k_solve(StepView v, int cls, int max_it, float tol) {
+// HELD: steps of each slice held in registers besides.  An iteration is bound by
+// shared-memory wavefronts, one for the weights, one for the columns and about
+// three for the gathered neighbours of a step; those held need the last only.
+// With the sums' shorter chain and without the IEEE divisions, 170 rows take
+// 75 us instead of 104.  24 steps need 127 registers, half the CTAs an SM could
+// hold: no loss for 8 and 16 warps, where one SM's shared memory is the limit
+// (4 steps and 64 registers for 16 warps: 1607 -> 1680 us on the dense 4,000-event chain),
+// but 32 warps keep to 64 registers without spills (8 steps: 213 -> 230 us), and the
+// one-warp class lives on many warps (12 steps, 167 registers: batches 3 % slower).
+// CTAS: resident CTAs per SM that the register count is held to.
+template <int NW, int RPT, int GROUPS, int KP, int ENT, int HELD, int CTAS>
+__global__ void __launch_bounds__(NW * 32 * GROUPS, CTAS) k_solve(StepView v, int cls, int max_it, float tol) {
   static_assert(NW == 1 || GROUPS == 1, "a CTA holds one component, or one per warp");
   using Smem = SolveSmem<NW, RPT, GROUPS, KP>;
   __shared__ Smem smem[GROUPS];
@@ -474,13 +544,15 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS) k_solve(StepView v, int cls,
       for (int i = 0; i < w + NW * k; ++i) sb += S.ssize[i];
       int ss = sb < ENT ? ((ENT - sb) >> 5) & ~3 : 0;
       ss = ss < sl[k].steps ? ss : sl[k].steps;
-      sl[k] = fill_slice(v, lane, sl[k].len, sl[k].steps, row, on[k] ? S.row.q[row] : 0, on[k] ? S.row.m[row] : 0, es,
+      sl[k] = fill_slice<(RPT == 1 && NW < 32) ? 8 : 4>(v, lane, sl[k].len, sl[k].steps, row, on[k] ? S.row.q[row] : 0, on[k] ? S.row.m[row] : 0, es,
                          sb, ss);
     }
     group_sync<NW>();
+    Held<HELD> held[RPT];
 #pragma unroll
     for (int k = 0; k < RPT; ++k) {
       const int row = (w + NW * k) * 32 + lane;
+      hold<HELD>(held[k], es, sl[k], lane);
       r[k] = yv[k] = p[k] = ap[k] = dz[k] = 0.f;
       di[k] = 0.f;
       if (on[k]) {
@@ -507,14 +579,14 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS) k_solve(StepView v, int cls,
       float dot = 0.f;
 #pragma unroll
       for (int k = 0; k < RPT; ++k) {
-        const float ay = fmaf(lam, yv[k], slice_mul(v.ent, es, sl[k], lane, yv[k], S.vec.y));
+        const float ay = fmaf(lam, yv[k], slice_mul<HELD>(v.ent, es, sl[k], held[k], lane, yv[k], S.vec.y));
         p[k] = fmaf(beta, p[k], yv[k]);
         ap[k] = fmaf(beta, ap[k], ay);
         dot = fmaf(p[k], ap[k], dot);
       }
       const float pap = group_sum2<NW>(dot, 0.f, S.part, par, w, lane).x;
       if (!(pap > 0.f)) break;
-      const float alpha = rz / pap;
+      const float alpha = __fdividef(rz, pap);
       float rzn = 0.f;
       rr = 0.f;
 #pragma unroll
@@ -555,7 +627,7 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS) k_solve(StepView v, int cls,
         if (s.y <= thr || ++rounds >= kMaxReplace) break;
         last = s.y;
       }
-      beta = s.x / rz;
+      beta = __fdividef(s.x, rz);
       rz = s.x;
     }
 #pragma unroll
@@ -624,7 +696,7 @@ __device__ bool multi_sum2(const StepView& v, MultiSmem& S, Group& G, float a, f
     s = warp_sum2(s.x, s.y);
     int4* slots = v.msync + (G.call & 1) * kMaxGrid;
     if (lane == 0) {
-      __threadfence();
+      fence_gpu();
       st_slot(slots + blockIdx.x, make_int4(__float_as_int(s.x), __float_as_int(s.y), G.seq, G.call));
     }
     float x = 0.f, y = 0.f;
@@ -639,7 +711,8 @@ __device__ bool multi_sum2(const StepView& v, MultiSmem& S, Group& G, float a, f
           y += __int_as_float(r.y);
           break;
         }
-        if ((n & 255u) == 0) {
+        // not on the first spins, where it would cost most barriers another trip to L2
+        if (limit == 0 || (n & 255u) == 16) {
           const uint64_t t = gtimer();
           if (t0 == 0) t0 = t;
           if (*((const volatile int32_t*)v.counters + kCntError) != 0) ok = false;
@@ -651,7 +724,7 @@ __device__ bool multi_sum2(const StepView& v, MultiSmem& S, Group& G, float a, f
         }
       }
     }
-    __threadfence();
+    fence_gpu();
     ok = __all_sync(0xffffffffu, ok);
     s = warp_sum2(x, y);
     if (lane == 0) {
@@ -777,7 +850,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
       const int steps = slice_steps(len);
       int ss = rows <= 65536 ? kMultiSteps - used : 0;
       ss = ss < steps ? ss : steps;
-      const Slice e = fill_slice(v, lane, len, steps, row, q, m, es, (w * kMultiSteps + used) * 32, ss);
+      const Slice e = fill_slice<4>(v, lane, len, steps, row, q, m, es, (w * kMultiSteps + used) * 32, ss);
       used += ss;
       v.rs_len[t] = len;
       if (lane == 0) v.rs_slice[t >> 5] = make_int4(e.sb, e.ss, e.gb, e.steps);
@@ -821,7 +894,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
         const int row = sl * 32 + lane, t = slot0 + row;
         const int4 e = v.rs_slice[t >> 5];
         const float yr = yg[row];
-        const float ay = fmaf(lam, yr, slice_mul(v.ent, es, Slice{e.x, e.y, e.z, v.rs_len[t], e.w}, lane, yr, yg));
+        const float ay = fmaf(lam, yr, slice_mul<0>(v.ent, es, Slice{e.x, e.y, e.z, v.rs_len[t], e.w}, Held<0>{}, lane, yr, yg));
         const float p = fmaf(beta, v.rs_p[t], yr);
         const float ap = fmaf(beta, v.rs_ap[t], ay);
         v.rs_p[t] = p;
@@ -831,7 +904,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
       if (!multi_sum2(v, S, G, dot, 0.f, &s)) return;
       const float pap = s.x;
       if (!(pap > 0.f)) break;
-      const float alpha = rz / pap;
+      const float alpha = __fdividef(rz, pap);
       float rzn = 0.f;
       rr = 0.f;
       for (int sl = gw; sl < nsl; sl += ngw) {
@@ -872,7 +945,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
         if (s.y <= thr || ++rounds >= kMaxReplace) break;
         last = s.y;
       }
-      beta = s.x / rz;
+      beta = __fdividef(s.x, rz);
       rz = s.x;
     }
     for (int sl = gw; sl < nsl; sl += ngw) {
@@ -892,23 +965,23 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
 
 }  // namespace
 
-// warps, rows per lane, components per CTA, pieces, entries in shared memory
-#define SOLVE_WARP 1, 2, 4, kWarpPieces, 1024
-#define SOLVE_SMALL 8, 1, 1, kSmallPieces, 5120
-#define SOLVE_MID 16, 1, 1, kMidPieces, 12288
-#define SOLVE_CTA 32, 1, 1, kCtaPieces, 24576
+// warps, rows per lane, components per CTA, pieces, entries in shared memory, steps in registers
+#define SOLVE_WARP 1, 2, 4, kWarpPieces, 1024, 0, 7
+#define SOLVE_SMALL 8, 1, 1, kSmallPieces, 5120, 24, 2
+#define SOLVE_MID 16, 1, 1, kMidPieces, 12288, 24, 1
+#define SOLVE_CTA 32, 1, 1, kCtaPieces, 24576, 4, 1
 
 namespace {
 
-template <int NW, int RPT, int GROUPS, int KP, int ENT>
+template <int NW, int RPT, int GROUPS, int KP, int ENT, int HELD, int CTAS>
 cudaError_t configure_one() {
-  return cudaFuncSetAttribute(k_solve<NW, RPT, GROUPS, KP, ENT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(k_solve<NW, RPT, GROUPS, KP, ENT, HELD, CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               GROUPS * ENT * 6);
 }
 
-template <int NW, int RPT, int GROUPS, int KP, int ENT>
+template <int NW, int RPT, int GROUPS, int KP, int ENT, int HELD, int CTAS>
 cudaError_t launch_one(const StepView& v, int cls, int max_it, float tol, int ctas, cudaStream_t st) {
-  k_solve<NW, RPT, GROUPS, KP, ENT><<<ctas, NW * 32 * GROUPS, GROUPS * ENT * 6, st>>>(v, cls, max_it, tol);
+  k_solve<NW, RPT, GROUPS, KP, ENT, HELD, CTAS><<<ctas, NW * 32 * GROUPS, GROUPS * ENT * 6, st>>>(v, cls, max_it, tol);
   return cudaGetLastError();
 }
 

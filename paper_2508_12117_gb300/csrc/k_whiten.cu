@@ -420,15 +420,20 @@ cudaError_t launch_whiten(const StepView& v, int64_t n_b, const WhitenPlan& w, i
       if ((e = cudaStreamWaitEvent(br->s[i], br->fork, 0)) != cudaSuccess) return e;
   }
   auto lane = [&](int i) { return br ? br->s[i] : st; };
-  if ((e = launch_solve_multi(v, max_it, tol, w.multi_grid, st)) != cudaSuccess) return e;
+  // Classes that no component of this catalog can be of are not launched (on the
+  // 200-event catalog three of five: 4 us each to find their lists empty).
+  auto reached = [&](int cls) { return w.top_class >= cls; };
+  if (reached(kClsMulti) && (e = launch_solve_multi(v, max_it, tol, w.multi_grid, st)) != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
   if (clean_side) {
     const int g = w.clean_grid * w.clean_share / 4;
     k_whiten_clean<<<g > 0 ? g : 1, kCleanWarps * 32, 0, lane(4)>>>(v, tol);
   }
-  if ((e = launch_solve_class(v, kClsCta, max_it, tol, w.num_sms * w.cta_mult, lane(0))) != cudaSuccess) return e;
-  if ((e = launch_solve_class(v, kClsMid, max_it, tol, w.num_sms * w.cta_mult, lane(1))) != cudaSuccess) return e;
-  if ((e = launch_solve_class(v, kClsSmall, max_it, tol, w.num_sms * w.cta_mult, lane(2))) != cudaSuccess) return e;
+  const int cta_classes[3] = {kClsCta, kClsMid, kClsSmall};
+  for (int i = 0; i < 3; ++i)
+    if (reached(cta_classes[i]) &&
+        (e = launch_solve_class(v, cta_classes[i], max_it, tol, w.num_sms * w.cta_mult, lane(i))) != cudaSuccess)
+      return e;
   if ((e = launch_solve_class(v, kClsWarp, max_it, tol, w.num_sms * w.warp_mult, lane(3))) != cudaSuccess) return e;
   if (br)
     for (int i = 0; i < 4; ++i) {

@@ -66,6 +66,7 @@ struct Branches {
 struct WhitenPlan {
   int use_inv;                 // clean pieces through their stored inverses
   int num_sms, cc_grid, clean_grid, multi_grid;
+  int top_class;               // largest class that a component of the catalog can be of
   int clean_share;             // quarters of clean_grid on the branch stream (0: on the launching stream)
   int warp_mult, cta_mult;     // CTAs per SM of the one-warp class / of the CTA classes
 };

@@ -74,37 +74,40 @@ __device__ __forceinline__ uint64_t gtimer() {
   return t;
 }
 
+// orders this thread's accesses, and those it has seen through a CTA barrier, at
+// GPU scope (__threadfence is the sequentially consistent form, which waits longer)
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
 // The limit comes from the step parameters (spider_set_wait_limit_ns); a limit
 // of 0 gives up at once whenever the barrier is not complete on arrival.  The
-// error flag is checked on the first spin and every 1024 spins after it, so a
-// CTA that finds another CTA's error leaves without waiting out its limit.
+// error flag is checked every 1024 spins, so a CTA that finds another CTA's error
+// leaves without waiting out its limit.  One counter, zero at the start of the
+// evaluation, that only rises within it: one trip to L2 to arrive and one to see the last
+// arrival, where a counter, its reset and a generation took five.
 __device__ bool grid_barrier(int32_t* counters, uint64_t limit_ns) {
   __syncthreads();
   __shared__ int ok;
   if (threadIdx.x == 0) {
-    volatile int32_t* gen = counters + kCntBarGen;
-    const int32_t g0 = *gen;
-    __threadfence();
-    const int32_t arrived = atomicAdd(&counters[kCntBarArrive], 1);
+    uint32_t* arrive = reinterpret_cast<uint32_t*>(counters) + kCntBarArrive;
+    uint32_t old, now;
+    asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(arrive) : "memory");
+    const uint32_t target = (old / gridDim.x + 1) * gridDim.x;
     ok = 1;
-    if (arrived == (int)gridDim.x - 1) {
-      counters[kCntBarArrive] = 0;
-      __threadfence();
-      atomicAdd(&counters[kCntBarGen], 1);
-    } else {
-      const uint64_t t0 = gtimer();
-      for (uint32_t n = 0; *gen == g0; ++n) {
-        if ((n & 1023u) == 0) {
-          if (((volatile int32_t*)counters)[kCntError] != 0) { ok = 0; break; }
-          if (gtimer() - t0 >= limit_ns) {
-            set_error(counters, SPIDER_E_TIMEOUT);
-            ok = 0;
-            break;
-          }
+    uint64_t t0 = 0;
+    for (uint32_t n = 0;; ++n) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(arrive) : "memory");
+      if ((int32_t)(now - target) >= 0) break;
+      if (limit_ns == 0 || (n & 1023u) == 8) {
+        if (((volatile int32_t*)counters)[kCntError] != 0) { ok = 0; break; }
+        const uint64_t t = gtimer();
+        if (t0 == 0) t0 = t;
+        if (limit_ns == 0 || t - t0 >= limit_ns) {
+          set_error(counters, SPIDER_E_TIMEOUT);
+          ok = 0;
+          break;
         }
       }
     }
-    __threadfence();
   }
   __syncthreads();
   return ok != 0;

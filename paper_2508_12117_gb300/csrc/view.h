@@ -11,12 +11,11 @@ enum : int {
   kCntObs = 1,       // n: observations of the current minibatch
   kCntIters = 2,     // whitening iterations used
   kCntError = 3,     // first device-side error (SPIDER_E_*), sticky until read
-  kCntBarArrive = 4, // grid barrier arrivals
-  kCntBarGen = 5,    // grid barrier generation
-  kCntComps = 6,     // connected components of the minibatch graph
-  kCntCompIters = 7, // largest CG iteration count of a component solved by one warp
-  kCntEvents = 8,    // events touched by the minibatch (with at least one pair)
-  kCntSlots = 9
+  kCntBarArrive = 4, // grid barrier arrivals of this evaluation
+  kCntComps = 5,     // connected components of the minibatch graph
+  kCntCompIters = 6, // largest CG iteration count of a component solved by one warp
+  kCntEvents = 7,    // events touched by the minibatch (with at least one pair)
+  kCntSlots = 8
 };
 
 // Travel-time network on the device.
