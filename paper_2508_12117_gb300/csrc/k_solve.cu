@@ -664,17 +664,23 @@ struct Group {
   int rank, size, cta0;
 };
 
+// A word is one 128-bit access: the sums must be those of the barrier number read
+// with them, and a vector access (.v4.s32) is four accesses in no stated order.
 __device__ __forceinline__ int4 ld_slot(const int4* p) {
-  int4 r;
-  asm volatile("ld.volatile.global.v4.s32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
-               : "l"(p)
-               : "memory");
-  return r;
+  uint64_t a, b;
+  asm volatile(
+      "{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+      : "=l"(a), "=l"(b)
+      : "l"(p)
+      : "memory");
+  return make_int4((int)a, (int)(a >> 32), (int)b, (int)(b >> 32));
 }
 __device__ __forceinline__ void st_slot(int4* p, int4 r) {
-  asm volatile("st.volatile.global.v4.s32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(r.x), "r"(r.y), "r"(r.z), "r"(r.w)
-               : "memory");
+  const uint64_t a = (uint32_t)r.x | (uint64_t)(uint32_t)r.y << 32, b = (uint32_t)r.z | (uint64_t)(uint32_t)r.w << 32;
+  asm volatile(
+      "{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p),
+      "l"(a), "l"(b)
+      : "memory");
 }
 
 // Group-wide barrier with two sums (fixed order).  Each CTA publishes its sums
