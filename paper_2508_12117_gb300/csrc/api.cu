@@ -9,6 +9,7 @@
 
 #include "kernels.h"
 #include "pieces.h"
+#include "pool.h"
 #include "prep.h"
 #include "spider.h"
 
@@ -474,8 +475,7 @@ int build_whitening(spider_ctx* c, const Prep& P, bool want_inverses) {
   if ((e = cudaMemsetAsync(v.wfast, 0, (kWSlots + 64) * sizeof(int32_t), st))) return cuda_fail(c, e, "memset");
   ALF(rowof, PP);
   ALF(mrow, Q);
-  // entries of the largest step: two per selected observation, at most as much padding
-  ALF(ent, 4 * (size_t)P.N);
+  ALF(ent, (size_t)pool_entries(P.N, P.P));
   {
     // rows of the multi-CTA class in whole slices: such a unit has more than
     // kCtaRows rows, or more than kCtaPieces pieces

@@ -28,6 +28,7 @@
 
 #include "dfloat.cuh"
 #include "kernels.h"
+#include "pool.h"
 #include "step_util.cuh"
 
 namespace spider {
@@ -46,8 +47,8 @@ constexpr int kMultiThreads = 512;   // threads per CTA of the multi-CTA class
 
 // Where the entries of a slice are.  Steps [0, ss) sit in shared memory from sb
 // on, 32 words a step (rows shorter than `steps` padded with zero weights, so
-// the loop needs no predicate); the other steps in the pool in global memory:
-// padded the same way from gb on (gb >= 0), or from ~gb on with the t-th entries
+// the loop needs no predicate); the other steps in the pool in global memory from
+// pool_first(gb) on: padded the same way (gb >= 0), or with the t-th entries
 // of the rows that have one side by side (slices of very uneven rows, where
 // padding would more than double the entries).  ss and steps are multiples of 4.
 struct Slice {
@@ -87,13 +88,15 @@ __device__ __forceinline__ Slice fill_slice(const StepView& v, int lane, int len
   }
   Slice s{sb, ss, 0, len, steps};
   const int rest = __reduce_add_sync(0xffffffffu, len > ss ? len - ss : 0);
-  const bool padded = 32 * (steps - ss) <= 2 * rest;
-  int at = 0;
+  const bool padded = pool_padded(steps - ss, rest);
   if (steps > ss) {
-    if (lane == 0) at = atomicAdd(&v.wfast[kWEntries], padded ? 32 * (steps - ss) : rest);
-    at = __shfl_sync(0xffffffffu, at, 0);
-    s.gb = padded ? at : ~at;
+    int g = 0;
+    if (lane == 0) g = atomicAdd(&v.wfast[kWEntries], pool_grains(steps - ss, rest));
+    g = __shfl_sync(0xffffffffu, g, 0);
+    s.gb = padded ? g : ~g;
   }
+  float2* const ent = v.ent + pool_first(s.gb);
+  int at = 0;                            // entries written, not padded
   // kFill entries at a time: three dependent trips to L2 each (8 instead of 4 saves a
   // tenth of a component's time); steps is a multiple of 4
   for (int j = 0; j < steps; j += kFill) {
@@ -103,7 +106,7 @@ __device__ __forceinline__ Slice fill_slice(const StepView& v, int lane, int len
       if (j + i < ss) {
         pos[i] = sb + 32 * (j + i) + lane;
       } else if (padded) {
-        pos[i] = at + 32 * (j - ss + i) + lane;
+        pos[i] = 32 * (j - ss + i) + lane;
       } else {
         const unsigned mask = __ballot_sync(0xffffffffu, j + i < len);
         pos[i] = at + __popc(mask & lt);
@@ -143,7 +146,7 @@ __device__ __forceinline__ Slice fill_slice(const StepView& v, int lane, int len
         es.sw[pos[i]] = sw[i];
         es.col[pos[i]] = (uint16_t)col[i];
       } else if (padded || j + i < len) {
-        v.ent[pos[i]] = make_float2(sw[i], __int_as_float(col[i]));
+        ent[pos[i]] = make_float2(sw[i], __int_as_float(col[i]));
       }
     }
   }
@@ -207,8 +210,9 @@ __device__ __forceinline__ float slice_mul(const float2* ent, EntrySmem es, cons
     }
   }
   if (sl.steps == sl.ss) return s;
+  ent += pool_first(sl.gb);
   if (sl.gb >= 0) {
-    const float2* p = ent + sl.gb + lane;
+    const float2* p = ent + lane;
     for (int j = sl.ss; j < sl.steps; j += 8, p += 8 * 32) {
       float2 x[8];
 #pragma unroll
@@ -219,7 +223,7 @@ __device__ __forceinline__ float slice_mul(const float2* ent, EntrySmem es, cons
     return s;
   }
   const unsigned lt = (1u << lane) - 1u;
-  int at = ~sl.gb;
+  int at = 0;
   for (int j = sl.ss; j < sl.steps; j += 4) {
     float2 x[4];
 #pragma unroll
@@ -253,7 +257,8 @@ __device__ __forceinline__ df32 slice_mul_df(const float2* ent, EntrySmem es, co
     for (int i = 0; i < 4; ++i) acc[i & 1] = df_add(acc[i & 1], t[i]);
   }
   const unsigned lt = (1u << lane) - 1u;
-  int at = sl.gb >= 0 ? sl.gb + lane : ~sl.gb;
+  ent += pool_first(sl.gb);
+  int at = sl.gb >= 0 ? lane : 0;
   for (int j = sl.ss; j < sl.steps; j += 4) {
     float2 x[4];
 #pragma unroll
@@ -412,6 +417,7 @@ __device__ void group_exscan(int32_t* a, int32_t* wsum, int tid, int w, int lane
 template <int NW, int RPT, int GROUPS, int KP, int ENT, int HELD, int CTAS>
 __global__ void __launch_bounds__(NW * 32 * GROUPS, CTAS) k_solve(StepView v, int cls, int max_it, float tol) {
   static_assert(NW == 1 || GROUPS == 1, "a CTA holds one component, or one per warp");
+  static_assert(ENT % 128 == 0, "whole groups of four steps");
   using Smem = SolveSmem<NW, RPT, GROUPS, KP>;
   __shared__ Smem smem[GROUPS];
   extern __shared__ __align__(16) uint8_t s_ent[];
@@ -533,7 +539,8 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS, CTAS) k_solve(StepView v, in
       on[k] = row < rows;
       sl[k] = Slice{0, 0, 0, on[k] ? S.row.len[row] : 0, 0};
       sl[k].steps = slice_steps(sl[k].len);
-      if (lane == 0) S.ssize[w + NW * k] = 32 * sl[k].steps;
+      // what it takes of shared memory, all of it at most (no sum overflows then)
+      if (lane == 0) S.ssize[w + NW * k] = 32 * (sl[k].steps < ENT / 32 ? sl[k].steps : ENT / 32);
     }
     group_sync<NW>();
 #pragma unroll

@@ -190,7 +190,7 @@ struct StepView {
   int32_t* wfast;                 // [kWSlots + 64] counters and cursors, then the labelling rounds' flags
   int32_t* rowof;                 // P: row of a unique pair inside its component
   int32_t* mrow;                  // Q: the same per member occurrence
-  float2* ent;                    // 4N: matrix entries (sqrt w, column) by slice, padding included
+  float2* ent;                    // pool_entries: matrix entries (sqrt w, column) by slice, padding included
   // row slots of the multi-CTA class
   int32_t *rs_u, *rs_m, *rs_q, *rs_len;
   int4* rs_slice;                 // per slice: where its entries are
@@ -238,7 +238,7 @@ enum : int {
   kWClean = 3,      // pieces solved with their stored inverse
   kWCursorC = 4,    // their work cursor
   kWRowSlots = 5,   // row slots taken by the multi-CTA class
-  kWEntries = 6,    // entries taken from the pool
+  kWEntries = 6,    // grains taken from the pool of entries
   kWClass0 = 8,     // units per class list
   kWCursor0 = 16,   // work cursors of the class lists
   kWSlots = 24
