@@ -467,6 +467,7 @@ int build_whitening(spider_ctx* c, const Prep& P, bool want_inverses) {
   ALF(unit_slot, G);
   ALF(msync, 2 * kMaxGrid);
   ALF(unit_pieces, G); ALF(unit_pblk, G); ALF(unit_prow, G); ALF(unit_pbase, G);
+  v.unit_first = v.pcount;
   ALF(cls_list, (size_t)kLists * G);
   v.cls_cap = (int64_t)G;
   ALF(clean_list, G);

@@ -182,7 +182,9 @@ struct StepView {
   int32_t *unit_off, *unit_np, *unit_fill, *unit_rows;   // G: per unit: piece list, pieces, fill cursor, rows
   int32_t* unit_slot;             // G: multi-CTA units: first row slot
   int4* msync;                    // 2 x kMaxGrid: barrier words of the multi-CTA class
-  int32_t *unit_pieces, *unit_pblk, *unit_prow, *unit_pbase;   // G: piece lists: id, block, rows, first row
+  int32_t *unit_pieces, *unit_pblk, *unit_prow;   // G: piece lists: id, block, rows
+  int32_t* unit_pbase;            // G: multi-CTA units: rows before the piece in its sorted run
+  int32_t* unit_first;            // G: the same in the unit (pcount's memory, done with when units are listed)
   int32_t* cls_list;              // kLists x cls_cap: units of each size class
   int64_t cls_cap;
   int32_t* clean_list;            // G: pieces of the step solved with their inverse
