@@ -407,8 +407,8 @@ __device__ void group_exscan(int32_t* a, int32_t* wsum, int tid, int w, int lane
 // HELD: steps of each slice held in registers besides.  An iteration is bound by
 // shared-memory wavefronts, one for the weights, one for the columns and about
 // three for the gathered neighbours of a step; those held need the last only.
-// With the sums' shorter chain and without the IEEE divisions, 170 rows take
-// 75 us instead of 104.  24 steps need 127 registers, half the CTAs an SM could
+// With the sums' shorter chain, 170 rows took 75 us instead of 104 (before the step
+// lengths were divided with IEEE rounding again, see below).  24 steps need 127 registers, half the CTAs an SM could
 // hold: no loss for 8 and 16 warps, where one SM's shared memory is the limit
 // (4 steps and 64 registers for 16 warps: 1607 -> 1680 us on the dense 4,000-event chain),
 // but 32 warps keep to 64 registers without spills (8 steps: 213 -> 230 us), and the
@@ -581,6 +581,9 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS, CTAS) k_solve(StepView v, in
     const float thr = kAim * tol * tol * bb;
     float last = s.y, beta = 0.f;
     rz = s.x;
+    // alpha and beta are IEEE quotients: an approximate one is zero for a divisor above
+    // 2^126, and a component of residuals near 1e18 never left z = 0 (small gradients,
+    // chains and batches take 0 to 2 % longer with them)
     while (bb > 0.f && it < max_it) {
       // p = y + beta p, A p = A y + beta A p
       float dot = 0.f;
@@ -593,7 +596,7 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS, CTAS) k_solve(StepView v, in
       }
       const float pap = group_sum2<NW>(dot, 0.f, S.part, par, w, lane).x;
       if (!(pap > 0.f)) break;
-      const float alpha = __fdividef(rz, pap);
+      const float alpha = __fdiv_rn(rz, pap);
       float rzn = 0.f;
       rr = 0.f;
 #pragma unroll
@@ -634,7 +637,7 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS, CTAS) k_solve(StepView v, in
         if (s.y <= thr || ++rounds >= kMaxReplace) break;
         last = s.y;
       }
-      beta = __fdividef(s.x, rz);
+      beta = __fdiv_rn(s.x, rz);
       rz = s.x;
     }
 #pragma unroll
@@ -1002,7 +1005,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
       if (!multi_sum2(v, S, G, dot, 0.f, &s)) return;
       const float pap = s.x;
       if (!(pap > 0.f)) break;
-      const float alpha = __fdividef(rz, pap);
+      const float alpha = __fdiv_rn(rz, pap);
       float rzn = 0.f;
       rr = 0.f;
       for (int sl = gw; sl < nsl; sl += ngw) {
@@ -1043,7 +1046,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
         if (s.y <= thr || ++rounds >= kMaxReplace) break;
         last = s.y;
       }
-      beta = __fdividef(s.x, rz);
+      beta = __fdiv_rn(s.x, rz);
       rz = s.x;
     }
     for (int sl = gw; sl < nsl; sl += ngw) {
