@@ -408,11 +408,12 @@ __device__ void group_exscan(int32_t* a, int32_t* wsum, int tid, int w, int lane
 // shared-memory wavefronts, one for the weights, one for the columns and about
 // three for the gathered neighbours of a step; those held need the last only.
 // With the sums' shorter chain, 170 rows took 75 us instead of 104 (before the step
-// lengths were divided with IEEE rounding again, see below).  24 steps need 127 registers, half the CTAs an SM could
-// hold: no loss for 8 and 16 warps, where one SM's shared memory is the limit
-// (4 steps and 64 registers for 16 warps: 1607 -> 1680 us on the dense 4,000-event chain),
-// but 32 warps keep to 64 registers without spills (8 steps: 213 -> 230 us), and the
-// one-warp class lives on many warps (12 steps, 167 registers: batches 3 % slower).
+// lengths were divided with IEEE rounding again, see below).  24 steps need 127
+// registers, half the CTAs an SM could hold: no loss for 8 and 16 warps, where one
+// SM's shared memory is the limit (4 steps and 64 registers for 16 warps: 1607 ->
+// 1680 us on the dense 4,000-event chain), but 32 warps keep to 64 registers (8 steps
+// spill: 213 -> 230 us), and the one-warp class lives on many warps (12 steps, 167
+// registers: batches 3 % slower).
 // CTAS: resident CTAs per SM that the register count is held to.
 template <int NW, int RPT, int GROUPS, int KP, int ENT, int HELD, int CTAS>
 __global__ void __launch_bounds__(NW * 32 * GROUPS, CTAS) k_solve(StepView v, int cls, int max_it, float tol) {

@@ -16,6 +16,7 @@
 
 #include "dfloat.cuh"
 #include "kernels.h"
+#include "mlp32.h"
 #include "pairs.cuh"
 #include "spider.h"
 
@@ -66,24 +67,6 @@ __global__ void k_tt_gradient(NetView net, PairSource src, TTOut out) {
 }
 
 // ------------------------------------------------------------------ FP32 MLP
-constexpr int kTP = 64;       // pairs per tile (wide form; the narrow form takes 32)
-constexpr int kKC = 8;        // weight rows per staged chunk
-constexpr int kStagesW = 3;   // chunks in flight
-constexpr int kGroups = 8;    // partial sums over the hidden units: eight contiguous groups
-
-// The narrow form: CTAs per SM (one, where two would leave a thread too few
-// registers), and tiles of 32 pairs per SM up to which it is the faster form:
-// 4864 pairs (one a SM) take 73 against 92 us at H = 128, 192 against 198 at 256;
-// two a SM 55 against 71 us at H = 64, but 123 against 120 at H = 128; four a SM
-// 44 against 66 us at H = 32.
-constexpr int narrow_ctas(int H) { return H >= 64 ? 1 : 4; }
-constexpr int narrow_tiles(int H) { return H >= 128 ? 1 : H >= 64 ? 2 : 4; }
-
-// CTAs per SM of the wide form's persistent grid: what registers (64 accumulators
-// a thread, 128 registers) and shared memory (the activations of a tile and three
-// weight chunks) hold
-__host__ __device__ constexpr int mlp_fp32_ctas(int H) { return H >= 256 ? 2 : H >= 128 ? 4 : H >= 64 ? 6 : 11; }
-
 __device__ __forceinline__ void silu_fp32(float z, float& h, float& ds) {
   const float s = 1.0f / (1.0f + expf(-z));
   h = z * s;
@@ -127,22 +110,7 @@ __device__ __forceinline__ void copy16(void* dst, const void* src) {
 // goes to a per-CTA scratch slot (rewritten every tile, so it stays in L2).
 // 300,000 pairs at H = 256: 8.41 -> 4.93 ms (28 -> 48 TFLOP/s of the 80 the FP32
 // lanes could do); 250,007 at H = 128: 1.58 -> 1.14 ms; 47 at H = 64: 47 -> 38 us.
-template <int H, bool WIDE>
-struct Mlp32 {
-  static constexpr int kPl = WIDE ? 2 : 1;           // pairs per lane
-  static constexpr int kUw = WIDE ? 32 : 8;          // units per warp
-  static constexpr int kTile = 32 * kPl;             // pairs per tile
-  static constexpr int kThreads = H / kUw * 32;
-  static constexpr int kChunkW = kKC * H;            // weights of a chunk
-  static constexpr int kTotal = 6 * (H / kKC);       // chunks per tile
-  static constexpr int kCtas = WIDE ? mlp_fp32_ctas(H) : narrow_ctas(H);
-  static constexpr int kUpg = H / kGroups;           // units per partial sum
-  static constexpr int kHold = WIDE ? 0 : H * kTile; // h4, kept for the sums of the narrow form
-  // act, weight chunks, inputs, partial sums [kGroups][4][kTile], h4
-  static constexpr size_t kSmem =
-      (size_t)(H * kTile + kStagesW * kChunkW + 6 * kTile + kGroups * 4 * kTile + kHold) * sizeof(float);
-};
-
+// The shapes are in mlp32.h.
 template <int PL>
 struct Lanes {
   float v[PL];
@@ -404,7 +372,7 @@ template <int H>
 cudaError_t launch_mlp_fp32(const NetView& net, const PairSource& src, TTOut out, int num_sms, int ctas_per_sm,
                             float* scratch, cudaStream_t st) {
   // never above the scratch slots
-  if (src.n_host <= (int64_t)32 * narrow_tiles(H) * num_sms)
+  if (narrow_form(H, src.n_host, num_sms))
     return launch_form<H, false>(net, src, out, narrow_ctas(H) * num_sms, scratch, st);
   return launch_form<H, true>(net, src, out, (ctas_per_sm == 1 ? 1 : mlp_fp32_ctas(H)) * num_sms, scratch, st);
 }
