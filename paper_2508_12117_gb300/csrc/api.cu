@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "kernels.h"
+#include "mlp32.h"
 #include "pieces.h"
 #include "pool.h"
 #include "prep.h"
@@ -266,7 +267,7 @@ cudaError_t step_sequence(spider_ctx* c, int64_t n_b, bool logpost, bool timed) 
   src.sta_hi = v.sta_hi;
   src.sta_lo = v.sta_lo;
   src.n_dev = v.counters + kCntPairs;
-  src.n_host = v.P;
+  src.n_host = step_pairs(v.P, n_b, v.L_max);
   TTOut out{v.T2, v.J, nullptr, nullptr};
   TRY(launch_tt(c->net, src, out, c->num_sms, c->tt_scratch, st, c->knobs[2]));
   if (timed) TRY(cudaEventRecord(c->ev[2], st));

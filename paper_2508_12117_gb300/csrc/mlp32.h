@@ -26,6 +26,12 @@ constexpr int narrow_tiles(int H) { return H >= 128 ? 1 : H >= 64 ? 2 : 4; }
 // 1,000,000 pairs: 804 us with eleven, 672 with ten)
 constexpr int mlp_fp32_ctas(int H) { return H >= 256 ? 2 : H >= 128 ? 4 : H >= 64 ? 6 : 10; }
 
+// Pairs of a step of n_b blocks, each of at most `nodes` pairs, in a catalog of P, at
+// most.  (By the catalog's pairs alone, a small minibatch of a large catalog took the
+// wide form and left SMs without a tile: a step of 1,000 pairs took 143 us at H = 64,
+// 171 at 128 and 480 at 256, now 115, 151 and 270.)
+constexpr int64_t step_pairs(int64_t P, int64_t n_b, int64_t nodes) { return n_b * nodes < P ? n_b * nodes : P; }
+
 // whether a launch of at most n pairs takes the narrow form
 constexpr bool narrow_form(int H, int64_t n, int num_sms) { return n <= (int64_t)32 * narrow_tiles(H) * num_sms; }
 

@@ -26,3 +26,7 @@ extern "C" int mlp32_shape(int H, int wide, long long* out) {
     default: return -1;
   }
 }
+
+extern "C" int mlp32_step_is_narrow(int H, long long P, long long n_b, long long nodes, int sms) {
+  return spider::narrow_form(H, spider::step_pairs(P, n_b, nodes), sms);
+}
