@@ -360,8 +360,13 @@ class Context:
         return dict(zip(names, list(ms))), ev.value
 
     def spider_last_whiten_timing(self):
-        """Device ms of the whitening phases of the last timed evaluation (see
-        include/spider.h); zeros unless it took the piece-inverse path."""
+        """Device ms of the whitening phases of the last timed evaluation (zeros
+        without whitening; see include/spider.h).  What the names stand for:
+        "pieces" labels and lists the components, "unit_setup" is always zero,
+        "unit_rounds" are the components held by one warp or one CTA (beyond the
+        next), "cta_passes" those spread over several CTAs, "clean_wait" the wait
+        for the stored inverses' kernel, "general" the pieces whose stored inverse
+        did not converge."""
         ms = (C.c_float * 6)()
         _check(load_library().spider_last_whiten_timing(self.h, ms), self.h)
         names = ["pieces", "unit_setup", "unit_rounds", "cta_passes", "clean_wait", "general"]
@@ -385,6 +390,10 @@ class Context:
         _check(load_library().spider_set_tuning(self.h, _ptr(arr, C.c_int32), arr.size), self.h)
 
     def spider_info(self):
+        """Facts about the context (see include/spider.h).  "units" are the
+        components left to conjugate gradients, "units_global" those of several
+        CTAs, "fallback" is 1 if there was one or a stored inverse did not converge;
+        the unit_kcycles_*, pass*_* and handover_* entries are always zero."""
         out = np.zeros(39, np.int64)
         _check(load_library().spider_info(self.h, _ptr(out, C.c_int64), 39), self.h)
         keys = ["n_sub", "graph", "blocks_per_step", "blocks", "pairs", "events", "obs", "components",

@@ -735,7 +735,6 @@ int create_impl(const spider_catalog* cat, const spider_stations* sta, const spi
   AL(estamp, M);
   AL(grad, M);
   AL(counters, kCntSlots);
-  AL(red, 8 * kMaxGrid);
   AL(dblk, NB);
   AL(dred, 4 * kMaxGrid);
   AL(dout, 8);

@@ -9,11 +9,11 @@ namespace spider {
 enum : int {
   kCntPairs = 0,     // P_u: unique pairs of the current minibatch
   kCntObs = 1,       // n: observations of the current minibatch
-  kCntIters = 2,     // whitening iterations used
+  kCntIters = 2,     // largest CG iteration count of a component on several CTAs
   kCntError = 3,     // first device-side error (SPIDER_E_*), sticky until read
   kCntBarArrive = 4, // grid barrier arrivals of this evaluation
   kCntComps = 5,     // connected components of the minibatch graph
-  kCntCompIters = 6, // largest CG iteration count of a component solved by one warp
+  kCntCompIters = 6, // largest CG iteration count of a component on one warp or CTA, or rounds of a stored inverse
   kCntEvents = 7,    // events touched by the minibatch (with at least one pair)
   kCntSlots = 8
 };
@@ -155,7 +155,6 @@ struct StepView {
   int32_t* estamp;
   float4* grad;
   int32_t* counters;
-  float* red;        // float reduction partials (whitening), 8 x kMaxGrid
   double* dblk;      // FP64 sum r^2 per selected block (NB)
   double* dred;      // FP64 diagnostics partials, 4 x kMaxGrid
   double* dout;      // FP64 results: [0] loglik (scaled), [1] logprior, [2] logcen, [3] logpost
