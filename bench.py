@@ -148,9 +148,9 @@ def hbm_bytes(n_obs, q_nodes, p_u, M, touched, pairs_per_event, sampled):
     """Algorithmic DRAM bytes per launch of the HBM-bound step kernels (every
     array element the kernel must read or write once):
       k_resid   20 B per observation (packed local indices, reduced dt, sqrt w,
-                the residual written, two half-edge codes) + 47 B per local node
+                the residual written, two half-edge codes) + 39 B per local node
                 (unique index, T hi/lo, pair, event, origin time, half-edge
-                start, multi flag, u hi/lo, diagonal, row length, row offset);
+                start, multi flag, u hi/lo, diagonal);
       k_final   20 B per observation (indices, sqrt w, residual, q written,
                 half-edge codes) + 19 B per local node (unique index, z hi/lo,
                 half-edge start, multi flag, node sum written);
@@ -161,7 +161,7 @@ def hbm_bytes(n_obs, q_nodes, p_u, M, touched, pairs_per_event, sampled):
                 touched event its pair range and stamps (8 + 4 per pair) and
                 16 B per pair contribution."""
     return {
-        "k_resid": 20.0 * n_obs + 47.0 * q_nodes,
+        "k_resid": 20.0 * n_obs + 39.0 * q_nodes,
         "k_final": 20.0 * n_obs + 19.0 * q_nodes,
         "k_merge_s": 61.0 * p_u,
         "k_event": (44.0 + (16.0 if sampled else 0.0)) * M + touched * (8.0 + 4.0 * pairs_per_event)
