@@ -281,9 +281,24 @@ __device__ __forceinline__ df32 slice_mul_df(const float2* ent, EntrySmem es, co
   return df_add(acc[0], acc[1]);
 }
 
-// u - lambda z - B^T B z of one row, rounded to FP32
-__device__ __forceinline__ float row_residual(const StepView& v, int32_t u, df32 z, df32 bz) {
-  df32 rd = df_add(df32{v.rhs[u], v.rhs_lo[u]}, df_mul_f(z, -v.lam));
+// Power of two that a component's right-hand side is multiplied by, and its solution
+// divided by, from bb = |u|^2: one unless bb lies far out.  alpha and beta come from an
+// approximate division, good to 2 ulp for divisors in [2^-126, 2^126] and zero above: a
+// component of residuals near 1e18 never left z = 0.  (Its last bits steer the iteration
+// only, the residual is replaced in double-float: gradients are 1.4e-7 and 2.0e-7 from
+// 64 bits and chains 4.1e-11, 2.3e-11 and 9.5e-12, with IEEE quotients just as far, and
+// one chain 1.4e-11, with them 2.1e-11; chains and batches would take 1 to 2 % longer,
+// and as much with a test of every divisor.)
+__device__ __forceinline__ float rhs_scale(float bb) {
+  if (bb >= 0x1p-60f && bb <= 0x1p60f) return 1.f;
+  const int e = (int)(__float_as_uint(bb) >> 23 & 255u) - 127;
+  if (e == 128) return 0x1p-100f;                               // the squares do not fit FP32
+  return __uint_as_float((uint32_t)(127 - (e >> 1)) << 23);     // bb scale^2 in [1, 4)
+}
+
+// scale u - lambda z - B^T B z of one row, rounded to FP32
+__device__ __forceinline__ float row_residual(const StepView& v, int32_t u, float scale, df32 z, df32 bz) {
+  df32 rd = df_add(df32{scale * v.rhs[u], scale * v.rhs_lo[u]}, df_mul_f(z, -v.lam));
   rd = df_add(rd, df32{-bz.hi, -bz.lo});
   return rd.hi;
 }
@@ -366,6 +381,7 @@ struct SolveSmem {
   alignas(16) float2 part[2 * NW];
   int32_t wsum[NW], ssize[NW * RPT];
   int32_t unit;
+  float scale;
 };
 
 // Exclusive scan of a[0, N) over the group, N / (32 NW) consecutive values per
@@ -407,13 +423,12 @@ __device__ void group_exscan(int32_t* a, int32_t* wsum, int tid, int w, int lane
 // HELD: steps of each slice held in registers besides.  An iteration is bound by
 // shared-memory wavefronts, one for the weights, one for the columns and about
 // three for the gathered neighbours of a step; those held need the last only.
-// With the sums' shorter chain, 170 rows took 75 us instead of 104 (before the step
-// lengths were divided with IEEE rounding again, see below).  24 steps need 127
-// registers, half the CTAs an SM could hold: no loss for 8 and 16 warps, where one
-// SM's shared memory is the limit (4 steps and 64 registers for 16 warps: 1607 ->
-// 1680 us on the dense 4,000-event chain), but 32 warps keep to 64 registers (8 steps
-// spill: 213 -> 230 us), and the one-warp class lives on many warps (12 steps, 167
-// registers: batches 3 % slower).
+// With the sums' shorter chain and without IEEE divisions, 170 rows take 75 us instead
+// of 104.  24 steps need 127 registers, half the CTAs an SM could hold: no loss for 8
+// and 16 warps, where one SM's shared memory is the limit (4 steps and 64 registers for
+// 16 warps: 1607 -> 1680 us on the dense 4,000-event chain), but 32 warps keep to 64
+// registers (8 steps spill: 213 -> 230 us), and the one-warp class lives on many warps
+// (12 steps, 167 registers: batches 3 % slower).
 // CTAS: resident CTAs per SM that the register count is held to.
 template <int NW, int RPT, int GROUPS, int KP, int ENT, int HELD, int CTAS>
 __global__ void __launch_bounds__(NW * 32 * GROUPS, CTAS) k_solve(StepView v, int cls, int max_it, float tol) {
@@ -578,13 +593,24 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS, CTAS) k_solve(StepView v, in
     }
     int par = 0, it = 0, rounds = 0;
     bb = group_sum2<NW>(bb, 0.f, S.part, par, w, lane).x;
+    const float scale = rhs_scale(bb);
+    if (tid == 0) S.scale = scale;
+    if (scale != 1.f) {
+      rz = rr = 0.f;
+#pragma unroll
+      for (int k = 0; k < RPT; ++k) {
+        r[k] *= scale;
+        yv[k] = r[k] * di[k];
+        S.vec.y[(w + NW * k) * 32 + lane] = yv[k];
+        rz = fmaf(r[k], yv[k], rz);
+        rr = fmaf(r[k], r[k], rr);
+      }
+    }
     float2 s = group_sum2<NW>(rz, rr, S.part, par, w, lane);
+    if (scale != 1.f) bb = s.y;
     const float thr = kAim * tol * tol * bb;
     float last = s.y, beta = 0.f;
     rz = s.x;
-    // alpha and beta are IEEE quotients: an approximate one is zero for a divisor above
-    // 2^126, and a component of residuals near 1e18 never left z = 0 (small gradients,
-    // chains and batches take 0 to 2 % longer with them)
     while (bb > 0.f && it < max_it) {
       // p = y + beta p, A p = A y + beta A p
       float dot = 0.f;
@@ -597,7 +623,7 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS, CTAS) k_solve(StepView v, in
       }
       const float pap = group_sum2<NW>(dot, 0.f, S.part, par, w, lane).x;
       if (!(pap > 0.f)) break;
-      const float alpha = __fdiv_rn(rz, pap);
+      const float alpha = __fdividef(rz, pap);
       float rzn = 0.f;
       rr = 0.f;
 #pragma unroll
@@ -628,7 +654,7 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS, CTAS) k_solve(StepView v, in
           const int row = (w + NW * k) * 32 + lane;
           const df32 z = {S.vec.zh[row], S.vec.zl[row]};
           const df32 bz = slice_mul_df(v.ent, es, sl[k], lane, z, S.vec.zh, S.vec.zl);
-          r[k] = on[k] ? row_residual(v, u[k], z, bz) : 0.f;
+          r[k] = on[k] ? row_residual(v, u[k], S.scale, z, bz) : 0.f;
           yv[k] = r[k] * di[k];
           S.vec.y[row] = yv[k];
           rzn = fmaf(r[k], yv[k], rzn);
@@ -638,16 +664,17 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS, CTAS) k_solve(StepView v, in
         if (s.y <= thr || ++rounds >= kMaxReplace) break;
         last = s.y;
       }
-      beta = __fdiv_rn(s.x, rz);
+      beta = __fdividef(s.x, rz);
       rz = s.x;
     }
 #pragma unroll
     for (int k = 0; k < RPT; ++k)
       if (on[k]) {
         const int row = (w + NW * k) * 32 + lane;
+        const float back = 1.f / S.scale;                      // exact
         const df32 zn = df_add_f(df32{S.vec.zh[row], S.vec.zl[row]}, dz[k]);
-        v.z[u[k]] = zn.hi;
-        v.z_lo[u[k]] = zn.lo;
+        v.z[u[k]] = back * zn.hi;
+        v.z_lo[u[k]] = back * zn.lo;
       }
     if (it > most) most = it;
   }
@@ -674,6 +701,7 @@ static_assert(kRun * sizeof(uint64_t) <= kMultiBytes && kRun % kMultiThreads == 
 struct MultiSmem {
   float2 part[kMultiThreads / 32];
   float2 sum;
+  float scale;
   int32_t unit, size, ok;
   int32_t scan[33];
 };
@@ -978,7 +1006,21 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
     float2 s;
     if (!multi_sum2(v, S, G, bb, 0.f, &s)) return;
     bb = s.x;
+    const float scale = rhs_scale(bb);
+    if (tid == 0) S.scale = scale;
+    if (scale != 1.f) {
+      rz = rr = 0.f;
+      for (int sl = gw; sl < nsl; sl += ngw) {
+        const int row = sl * 32 + lane, t = slot0 + row;
+        const float r = scale * v.rs_r[t], yy = r * v.rs_di[t];
+        v.rs_r[t] = r;
+        y[row] = yy;
+        rz = fmaf(r, yy, rz);
+        rr = fmaf(r, r, rr);
+      }
+    }
     if (!multi_sum2(v, S, G, rz, rr, &s)) return;
+    if (scale != 1.f) bb = s.y;
     const float thr = kAim * tol * tol * bb;
     float last = s.y, beta = 0.f;
     rz = s.x;
@@ -1006,7 +1048,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
       if (!multi_sum2(v, S, G, dot, 0.f, &s)) return;
       const float pap = s.x;
       if (!(pap > 0.f)) break;
-      const float alpha = __fdiv_rn(rz, pap);
+      const float alpha = __fdividef(rz, pap);
       float rzn = 0.f;
       rr = 0.f;
       for (int sl = gw; sl < nsl; sl += ngw) {
@@ -1036,7 +1078,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
           const int4 e = v.rs_slice[t >> 5];
           const df32 z = {zh[row], zl[row]};
           const df32 bz = slice_mul_df(v.ent, es, Slice{e.x, e.y, e.z, v.rs_len[t], e.w}, lane, z, zh, zl);
-          const float r = row < rows ? row_residual(v, v.rs_u[t], z, bz) : 0.f;
+          const float r = row < rows ? row_residual(v, v.rs_u[t], S.scale, z, bz) : 0.f;
           const float yy = r * v.rs_di[t];
           v.rs_r[t] = r;
           y[row] = yy;
@@ -1047,7 +1089,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
         if (s.y <= thr || ++rounds >= kMaxReplace) break;
         last = s.y;
       }
-      beta = __fdiv_rn(s.x, rz);
+      beta = __fdividef(s.x, rz);
       rz = s.x;
     }
     for (int sl = gw; sl < nsl; sl += ngw) {
@@ -1055,8 +1097,9 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
       if (row >= rows) continue;
       const df32 zn = df_add_f(df32{zh[row], zl[row]}, v.rs_dz[t]);
       const int32_t u = v.rs_u[t];
-      v.z[u] = zn.hi;
-      v.z_lo[u] = zn.lo;
+      const float back = 1.f / S.scale;                        // exact
+      v.z[u] = back * zn.hi;
+      v.z_lo[u] = back * zn.lo;
     }
     // every word is read before the CTA's next group overwrites it
     if (!multi_sync(v, S, G)) return;
