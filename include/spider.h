@@ -302,7 +302,7 @@ int spider_debug_obs(spider_ctx *ctx, int64_t *idx_out, float *r_out, float *q_o
  * the FP32 MLP kernel (1..2), knobs[3] 1 (default): a piece (a block-local
  * component) that shares no node with another selected block is solved with
  * its stored inverse, where the inverses were built, 0: every component by
- * conjugate gradients; knobs[4] (0..4, default 1) the share, in quarters, of
+ * conjugate gradients; knobs[4] (0..4, default 2) the share, in quarters, of
  * the persistent grid the stored inverses' kernel takes on its branch stream
  * (0: it runs after the other components on the context's stream); knobs[5]
  * (1, 2 (default) or 4) threads per CTA of the per-block kernels (pair table,

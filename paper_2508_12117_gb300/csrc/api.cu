@@ -39,7 +39,7 @@ struct spider_ctx {
   cudaGraphExec_t graph_exec = nullptr;
   bool graph_ok = true;
   bool use_graph = true;
-  int32_t knobs[7] = {2, 1, 2, 1, 1, 2, 1};   // see spider_set_tuning
+  int32_t knobs[7] = {2, 1, 2, 1, 2, 2, 1};   // see spider_set_tuning
   // whitening: grids of its kernels, the branch streams of its size classes
   WhitenPlan plan{};
   bool inv = false;                // the pieces' inverses were built

@@ -426,10 +426,6 @@ cudaError_t launch_whiten(const StepView& v, int64_t n_b, const WhitenPlan& w, i
   if (reached(kClsMulti) && (e = launch_solve_multi(v, max_it, tol, w.multi_grid, st)) != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
   if (clean_side) {
-    // A quarter of its grid by default: with half of it the CTA classes wait for room
-    // on the SMs that its warps hold (1M-event BF16 step: 2.80 ms with half, 2.78 with
-    // a quarter, 2.82 with all of it or on the launching stream; batches and smaller
-    // catalogs within 0.5 % either way).
     const int g = w.clean_grid * w.clean_share / 4;
     k_whiten_clean<<<g > 0 ? g : 1, kCleanWarps * 32, 0, lane(4)>>>(v, tol);
   }
