@@ -256,6 +256,7 @@ __device__ __forceinline__ df32 slice_mul_df(const float2* ent, EntrySmem es, co
 #pragma unroll
     for (int i = 0; i < 4; ++i) acc[i & 1] = df_add(acc[i & 1], t[i]);
   }
+  if (sl.steps == sl.ss) return df_add(acc[0], acc[1]);
   const unsigned lt = (1u << lane) - 1u;
   ent += pool_first(sl.gb);
   int at = sl.gb >= 0 ? lane : 0;
@@ -281,8 +282,9 @@ __device__ __forceinline__ df32 slice_mul_df(const float2* ent, EntrySmem es, co
   return df_add(acc[0], acc[1]);
 }
 
-// Power of two that a component's right-hand side is multiplied by, and its solution
-// divided by, from bb = |u|^2: one unless bb lies far out.  alpha and beta come from an
+// Power of two that a component's right-hand side is multiplied by (in place: k_resid
+// writes it anew every step) and its solution divided by, from bb = |u|^2: one unless
+// bb lies far out.  alpha and beta come from an
 // approximate division, good to 2 ulp for divisors in [2^-126, 2^126] and zero above: a
 // component of residuals near 1e18 never left z = 0.  (Its last bits steer the iteration
 // only, the residual is replaced in double-float: gradients are 1.4e-7 and 2.0e-7 from
@@ -296,9 +298,9 @@ __device__ __forceinline__ float rhs_scale(float bb) {
   return __uint_as_float((uint32_t)(127 - (e >> 1)) << 23);     // bb scale^2 in [1, 4)
 }
 
-// scale u - lambda z - B^T B z of one row, rounded to FP32
-__device__ __forceinline__ float row_residual(const StepView& v, int32_t u, float scale, df32 z, df32 bz) {
-  df32 rd = df_add(df32{scale * v.rhs[u], scale * v.rhs_lo[u]}, df_mul_f(z, -v.lam));
+// u - lambda z - B^T B z of one row, rounded to FP32
+__device__ __forceinline__ float row_residual(const StepView& v, int32_t u, df32 z, df32 bz) {
+  df32 rd = df_add(df32{v.rhs[u], v.rhs_lo[u]}, df_mul_f(z, -v.lam));
   rd = df_add(rd, df32{-bz.hi, -bz.lo});
   return rd.hi;
 }
@@ -599,6 +601,10 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS, CTAS) k_solve(StepView v, in
       rz = rr = 0.f;
 #pragma unroll
       for (int k = 0; k < RPT; ++k) {
+        if (on[k]) {
+          v.rhs[u[k]] *= scale;
+          v.rhs_lo[u[k]] *= scale;
+        }
         r[k] *= scale;
         yv[k] = r[k] * di[k];
         S.vec.y[(w + NW * k) * 32 + lane] = yv[k];
@@ -654,7 +660,7 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS, CTAS) k_solve(StepView v, in
           const int row = (w + NW * k) * 32 + lane;
           const df32 z = {S.vec.zh[row], S.vec.zl[row]};
           const df32 bz = slice_mul_df(v.ent, es, sl[k], lane, z, S.vec.zh, S.vec.zl);
-          r[k] = on[k] ? row_residual(v, u[k], S.scale, z, bz) : 0.f;
+          r[k] = on[k] ? row_residual(v, u[k], z, bz) : 0.f;
           yv[k] = r[k] * di[k];
           S.vec.y[row] = yv[k];
           rzn = fmaf(r[k], yv[k], rzn);
@@ -671,10 +677,13 @@ __global__ void __launch_bounds__(NW * 32 * GROUPS, CTAS) k_solve(StepView v, in
     for (int k = 0; k < RPT; ++k)
       if (on[k]) {
         const int row = (w + NW * k) * 32 + lane;
-        const float back = 1.f / S.scale;                      // exact
         const df32 zn = df_add_f(df32{S.vec.zh[row], S.vec.zl[row]}, dz[k]);
-        v.z[u[k]] = back * zn.hi;
-        v.z_lo[u[k]] = back * zn.lo;
+        v.z[u[k]] = zn.hi;
+        v.z_lo[u[k]] = zn.lo;
+        if (S.scale != 1.f) {
+          v.z[u[k]] /= S.scale;
+          v.z_lo[u[k]] /= S.scale;
+        }
       }
     if (it > most) most = it;
   }
@@ -1012,6 +1021,10 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
       rz = rr = 0.f;
       for (int sl = gw; sl < nsl; sl += ngw) {
         const int row = sl * 32 + lane, t = slot0 + row;
+        if (row < rows) {
+          v.rhs[v.rs_u[t]] *= scale;
+          v.rhs_lo[v.rs_u[t]] *= scale;
+        }
         const float r = scale * v.rs_r[t], yy = r * v.rs_di[t];
         v.rs_r[t] = r;
         y[row] = yy;
@@ -1078,7 +1091,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
           const int4 e = v.rs_slice[t >> 5];
           const df32 z = {zh[row], zl[row]};
           const df32 bz = slice_mul_df(v.ent, es, Slice{e.x, e.y, e.z, v.rs_len[t], e.w}, lane, z, zh, zl);
-          const float r = row < rows ? row_residual(v, v.rs_u[t], S.scale, z, bz) : 0.f;
+          const float r = row < rows ? row_residual(v, v.rs_u[t], z, bz) : 0.f;
           const float yy = r * v.rs_di[t];
           v.rs_r[t] = r;
           y[row] = yy;
@@ -1097,9 +1110,12 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_solve_multi(StepView v, in
       if (row >= rows) continue;
       const df32 zn = df_add_f(df32{zh[row], zl[row]}, v.rs_dz[t]);
       const int32_t u = v.rs_u[t];
-      const float back = 1.f / S.scale;                        // exact
-      v.z[u] = back * zn.hi;
-      v.z_lo[u] = back * zn.lo;
+      v.z[u] = zn.hi;
+      v.z_lo[u] = zn.lo;
+      if (S.scale != 1.f) {
+        v.z[u] /= S.scale;
+        v.z_lo[u] /= S.scale;
+      }
     }
     // every word is read before the CTA's next group overwrites it
     if (!multi_sync(v, S, G)) return;
