@@ -97,9 +97,11 @@ __device__ __forceinline__ void copy16(void* dst, const void* src) {
 // each) a step of k.  The packed FMA runs at the FP32 rate with half the issue
 // slots, which leaves the other half to the loads: one 8-byte load of the lane's
 // two activations (doubled in registers) and eight 16-byte loads of the warp's 32
-// weights, the same for every lane, so ten shared-memory wavefronts against the
-// 16 cycles the FMAs take.  (Lanes of 8 pairs x 8 units need fewer loads but 16
-// wavefronts: a 16-byte load of distinct addresses takes four.)
+// weights, the same for every lane.  That is about 18 wavefronts of the SM's shared
+// memory against the 16 cycles its FMA lanes take (a 16-byte load takes two even where
+// all lanes read one address; counted at 250,007 pairs and H = 128: shared memory busy
+// 72 % of the time, FMA lanes 62 %), so shared memory is what bounds it, with 14 warps
+// an SM to overlap the two.
 // Narrow form, for launches that leave SMs without a tile: tiles of 32 pairs, a
 // lane one pair x 8 units, so a tile is spread over eight times the lanes.
 // Every output is one chain of fused multiply-adds over k in ascending order,

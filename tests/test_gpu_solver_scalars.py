@@ -1,7 +1,7 @@
-"""Step lengths of the conjugate gradients near the top of FP32 and beyond: residuals so large
-that p.Ap lies between 2^126 and 2^128, where an approximate division returns zero
-and a component never leaves its start.  Every size class, against the FP64 oracle,
-gates as in test_gpu_components."""
+"""Step lengths of the conjugate gradients near the top of FP32 and beyond: residuals
+so large that p.Ap lies between 2^126 and 2^128, where an approximate division
+returns zero and a component never leaves its start, and squares beyond FP32.  Every
+size class, against the FP64 oracle, gates as in test_gpu_components."""
 import numpy as np
 import pytest
 
